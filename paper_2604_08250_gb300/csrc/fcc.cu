@@ -441,38 +441,6 @@ __global__ void __launch_bounds__(256) k_fcc_qsro_ministep(const __grid_constant
     if (P.acc_out) P.acc_out[c] = acc ? 1 : 0;
 }
 
-// e_acc += sum of part_e, n_acc += sum of part_n, in a fixed order: thread t
-// sums link cells t, t + 1024, ... in turn, then a fixed pairwise tree over
-// the 1024 partial sums (one block of kFccReduceThreads).
-constexpr int kFccReduceThreads = 1024;
-__global__ void __launch_bounds__(kFccReduceThreads) k_fcc_reduce(const double *part_e, const long long *part_n, int n,
-                                                                  double *e_acc, long long *n_acc)
-{
-    __shared__ double se[kFccReduceThreads];
-    __shared__ long long sn[kFccReduceThreads];
-    const int t = threadIdx.x;
-    double e = 0.0;
-    long long c = 0;
-    for (int i = t; i < n; i += kFccReduceThreads) {
-        e += part_e[i];
-        c += part_n[i];
-    }
-    se[t] = e;
-    sn[t] = c;
-    __syncthreads();
-    for (int h = kFccReduceThreads / 2; h > 0; h >>= 1) {
-        if (t < h) {
-            se[t] += se[t + h];
-            sn[t] += sn[t + h];
-        }
-        __syncthreads();
-    }
-    if (t == 0) {
-        if (e_acc) *e_acc += se[0];
-        if (n_acc) *n_acc += sn[0];
-    }
-}
-
 // Ordered pair counts n_m^{pq} (each site's shell-m neighbours), per-block
 // shared counters flushed with 64-bit atomics.
 // With sq non-null also Q_m^p = sum over sites of species p of the squared
@@ -781,9 +749,9 @@ smc_status launch_fcc_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     std::vector<uint32_t> words;
     st = is_qsro ? fcc_qsro_tables(lat, m, words) : fcc_sweep_tables(lat, m, words);
     if (st != SMC_OK) return st;
-    // workspace: [part_e | part_n | ministep tables | acceptance tables | qSRO count cache]
+    // workspace: [part_e | part_n | ministep tables | acceptance tables | reduction scratch | qSRO count cache]
     const size_t off_pn = (size_t)nc * 8, off_w = off_pn + (size_t)nc * 8, off_tab = off_w + words.size() * 4;
-    const size_t off_q = (off_tab + tabs.size() * 4 + 255) / 256 * 256;
+    const size_t off_red = (off_tab + tabs.size() * 4 + 255) / 256 * 256, off_q = off_red + lc_reduce_bytes();
     const size_t N = 4ull * lat->nx * lat->ny * lat->nz;
     const size_t qbytes = m->nshells == 3 ? 2 : 1;
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, off_q + (is_qsro ? N * qbytes : 16), &st);
@@ -827,11 +795,8 @@ smc_status launch_fcc_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "k_fcc_ministep");
     }
-    if (e_acc || n_acc) {
-        k_fcc_reduce<<<1, kFccReduceThreads, 0, stream>>>(P.part_e, P.part_n, nc, e_acc, (long long *)n_acc);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return cuda_fail(e, "k_fcc_reduce");
-    }
+    if (e_acc || n_acc)
+        return launch_lc_reduce(P.part_e, P.part_n, nc, scr + off_red, e_acc, (long long *)n_acc, stream);
     return SMC_OK;
 }
 

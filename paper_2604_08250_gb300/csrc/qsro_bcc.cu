@@ -276,31 +276,46 @@ __global__ void __launch_bounds__(256) k_bq_ministep(const __grid_constant__ BqS
     if (P.acc_out) P.acc_out[c] = acc ? 1 : 0;
 }
 
-// e_acc += sum of part_e, n_acc += sum of part_n, in a fixed order.
-constexpr int kBqReduceThreads = 1024;
-__global__ void __launch_bounds__(kBqReduceThreads) k_bq_reduce(const double *part_e, const long long *part_n, int n,
-                                                                double *e_acc, long long *n_acc)
+// e_acc += sum of part_e, n_acc += sum of part_n, in a fixed order: block b
+// sums entries b * 1024 + t, + kLcBlocks * 1024, ... per thread and a pairwise
+// tree over its threads; the last block adds the blocks' sums the same way.
+// One block alone takes 8 bytes x 2 per entry at the latency of one SM (2.1 M
+// link cells at 512^3: over a millisecond).
+constexpr int kLcThreads = 1024, kLcBlocks = 128;
+
+__device__ __forceinline__ void lc_tree(double *se, long long *sn, int t)
 {
-    __shared__ double se[kBqReduceThreads];
-    __shared__ long long sn[kBqReduceThreads];
-    const int t = threadIdx.x;
-    double e = 0.0;
-    long long cnt = 0;
-    for (int i = t; i < n; i += kBqReduceThreads) {
-        e += part_e[i];
-        cnt += part_n[i];
-    }
-    se[t] = e;
-    sn[t] = cnt;
     __syncthreads();
-    for (int h = kBqReduceThreads / 2; h > 0; h >>= 1) {
+    for (int h = kLcThreads / 2; h > 0; h >>= 1) {
         if (t < h) {
             se[t] += se[t + h];
             sn[t] += sn[t + h];
         }
         __syncthreads();
     }
-    if (t == 0) {
+}
+
+__global__ void __launch_bounds__(kLcThreads) k_lc_sums(const double *part_e, const long long *part_n, long long n,
+                                                        double *out_e, long long *out_n, double *e_acc,
+                                                        long long *n_acc)
+{
+    __shared__ double se[kLcThreads];
+    __shared__ long long sn[kLcThreads];
+    const int t = threadIdx.x;
+    double e = 0.0;
+    long long cnt = 0;
+    for (long long i = (long long)blockIdx.x * kLcThreads + t; i < n; i += (long long)gridDim.x * kLcThreads) {
+        e += part_e[i];
+        cnt += part_n[i];
+    }
+    se[t] = e;
+    sn[t] = cnt;
+    lc_tree(se, sn, t);
+    if (t != 0) return;
+    if (out_e) {
+        out_e[blockIdx.x] = se[0];
+        out_n[blockIdx.x] = sn[0];
+    } else {
         if (e_acc) *e_acc += se[0];
         if (n_acc) *n_acc += sn[0];
     }
@@ -421,6 +436,25 @@ using BqKernel = void (*)(BqStep, int);
 
 }  // namespace
 
+size_t lc_reduce_bytes() { return (size_t)kLcBlocks * 16; }
+
+smc_status launch_lc_reduce(const double *part_e, const long long *part_n, long long n, void *scratch, double *e_acc,
+                            long long *n_acc, cudaStream_t stream)
+{
+    const long long blocks = std::min<long long>((n + kLcThreads - 1) / kLcThreads, kLcBlocks);
+    if (blocks > 1) {
+        double *e = (double *)scratch;
+        long long *c = (long long *)(e + kLcBlocks);
+        k_lc_sums<<<(int)blocks, kLcThreads, 0, stream>>>(part_e, part_n, n, e, c, nullptr, nullptr);
+        part_e = e;
+        part_n = c;
+        n = blocks;
+    }
+    k_lc_sums<<<1, kLcThreads, 0, stream>>>(part_e, part_n, n, nullptr, nullptr, e_acc, n_acc);
+    const cudaError_t err = cudaGetLastError();
+    return err == cudaSuccess ? SMC_OK : cuda_fail(err, "k_lc_sums");
+}
+
 smc_status launch_qsro_ministeps(const smc_lattice *lat, const smc_model *m, int8_t *occ, uint64_t seed,
                                  uint32_t replica, uint64_t sweep0, int nsweeps, const double *kT, double *e_acc,
                                  int64_t *n_acc, float *trace_dE, uint8_t *trace_acc, int trace_k,
@@ -452,8 +486,9 @@ smc_status launch_qsro_ministeps(const smc_lattice *lat, const smc_model *m, int
     std::vector<uint32_t> words;
     st = bq_tables(lat, m, words);
     if (st != SMC_OK) return st;
-    // workspace: [part_e | part_n | tables | count cache]
-    const size_t off_pn = (size_t)nc * 8, off_w = off_pn + (size_t)nc * 8, off_q = (off_w + words.size() * 4 + 255) / 256 * 256;
+    // workspace: [part_e | part_n | tables | reduction scratch | count cache]
+    const size_t off_pn = (size_t)nc * 8, off_w = off_pn + (size_t)nc * 8;
+    const size_t off_red = (off_w + words.size() * 4 + 255) / 256 * 256, off_q = off_red + lc_reduce_bytes();
     const size_t N = 2ull * lat->nx * lat->ny * lat->nz;
     const size_t qbytes = m->nshells == 3 ? 2 : 1;
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, off_q + N * qbytes, &st);
@@ -486,11 +521,8 @@ smc_status launch_qsro_ministeps(const smc_lattice *lat, const smc_model *m, int
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "k_bq_ministep");
     }
-    if (e_acc || n_acc) {
-        k_bq_reduce<<<1, kBqReduceThreads, 0, stream>>>(P.part_e, P.part_n, nc, e_acc, (long long *)n_acc);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return cuda_fail(e, "k_bq_reduce");
-    }
+    if (e_acc || n_acc)
+        return launch_lc_reduce(P.part_e, P.part_n, nc, scr + off_red, e_acc, (long long *)n_acc, stream);
     return SMC_OK;
 }
 

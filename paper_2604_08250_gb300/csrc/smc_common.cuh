@@ -186,6 +186,12 @@ smc_status launch_qsro_ministeps(const smc_lattice *lat, const smc_model *m, int
                                  uint32_t replica, uint64_t sweep0, int nsweeps, const double *kT, double *e_acc,
                                  int64_t *n_acc, float *trace_dE, uint8_t *trace_acc, int trace_k,
                                  cudaStream_t stream);
+// Sum of per-link-cell partial sums (part_e, part_n, n of each) into e_acc and
+// n_acc (either nullable), in a fixed order; scratch: lc_reduce_bytes() bytes
+// of device memory, 8-byte aligned (qsro_bcc.cu).
+size_t lc_reduce_bytes();
+smc_status launch_lc_reduce(const double *part_e, const long long *part_n, long long n, void *scratch, double *e_acc,
+                            long long *n_acc, cudaStream_t stream);
 smc_status launch_qsro_energy(const smc_lattice *lat, const smc_model *m, const int8_t *occ, double *e,
                               cudaStream_t stream);
 smc_status launch_qsro_grad(const smc_lattice *lat, const smc_model *m, const int8_t *occ, float *grad,
