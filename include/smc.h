@@ -162,7 +162,11 @@ smc_status smc_init_lattice(const smc_lattice *lat, const int64_t *counts, uint6
  * interaction zone of every accepted swap, so a trial evaluates only the 40
  * post-swap energies of its zone, and the per-site features (species and
  * per-shell species counts, 16 N bytes) the same way; they need every axis
- * a multiple of 4 cells and >= 8, nx <= 1024.  qSRO models keep each site's
+ * a multiple of 4 cells and >= 8, nx <= 1024.  A call that would evaluate
+ * more rows than there are feature vectors (9.5e8 for five species: about
+ * one sweep of 256^3) evaluates every vector once and looks the others up
+ * (8 N bytes and 4 bytes per vector of workspace; without room for them it
+ * runs as a smaller call does), with the same results bit for bit.  qSRO models keep each site's
  * own-species count per shell (N bytes for 1-2 shells, 2 N for 3), built at
  * the start of every call and updated by accepted swaps; a trial's dE comes
  * from the species of a, b and the sites within the model's shells of

@@ -25,172 +25,11 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <type_traits>
 #include <vector>
 
-#include "mlp_common.cuh"
-#include "mlp_tc.cuh"
-#include "mlpnet_tc.cuh"
-#include "sweep_common.cuh"
+#include "mlp_zone.cuh"
 
 namespace smc {
-
-constexpr int kOmega = 40;       // sites of a trial's interaction zone
-constexpr int kMlpChunk = 64;    // most trials of a mini-step evaluated together (40 rows each)
-constexpr int kTraceTB = 3;      // trials per trace step (120 rows: one tile)
-constexpr int kTcMaxCtasPerSm = 512 / (2 * kTcCols);  // for the 2-warpgroup kernels
-constexpr int kTinfo = 16;       // ints of per-trial information
-
-// Omega of a trial for each (trial sublattice, partner direction): rel = 0
-// for a site of the trial sublattice, 1 for the partner's; (dxo, dy, dz) its
-// cell offset from the trial site's cell.  Entry 0 is a, entry 1 is b.
-struct OmegaEntry {
-    signed char rel, dy, dz, dxo;
-    signed char ma, mb;  // shell (1-3) in which the site sees a / b, 0 if none
-    signed char pad[2];
-};
-struct MlpGeo {
-    OmegaEntry om[2][8][kOmega];
-};
-
-// Shared memory of the MLP kernels: weights, the warpgroups' tiles, then
-// kernel-specific parts from END on.
-template <int NWG>
-struct MlpSmem {
-    static constexpr uint32_t W1 = 0;
-    static constexpr uint32_t W2 = W1 + kTcW1;
-    static constexpr uint32_t X = W2 + kTcW2;        // [NWG] tiles
-    static constexpr uint32_t H = X + NWG * kTcX;    // [NWG] tiles
-    static constexpr uint32_t B1 = H + NWG * kTcH;
-    static constexpr uint32_t B2 = B1 + 256;
-    static constexpr uint32_t W3 = B2 + 256;
-    static constexpr uint32_t B3 = W3 + 256;
-    static constexpr uint32_t MBAR = B3 + 16;        // [NWG][2]
-    static constexpr uint32_t TSLOT = MBAR + 16 * NWG;
-    static constexpr uint32_t CTL = TSLOT + 4;       // CTA-wide flag
-    static constexpr uint32_t RED = (CTL + 4 + 15) / 16 * 16;  // 4 doubles / long longs for reductions
-    static constexpr uint32_t TINFO = RED + 64;      // int [kMlpChunk][kTinfo]
-    static constexpr uint32_t ACT = TINFO + kMlpChunk * kTinfo * 4;  // int [kMlpChunk]: trials with A != B
-    static constexpr uint32_t D = ACT + kMlpChunk * 4;  // pair table (kDEntries floats)
-    static constexpr uint32_t GEO = D + kDEntries * 4;
-    static constexpr uint32_t END = (uint32_t)((GEO + sizeof(MlpGeo) + 127) / 128 * 128);
-    static_assert(X % 128 == 0 && H % 128 == 0 && W2 % 128 == 0, "tile alignment");
-    static_assert(MBAR % 8 == 0 && RED % 8 == 0, "alignment");
-};
-constexpr int kSweepWG = 4;  // warpgroups of the sweep kernel (64-wide network)
-constexpr int kEvalWG = 2;   // warpgroups of the energy and trace kernels
-
-// Shared memory of the MLPNet kernels (96-wide, three ReLU layers): the same
-// kernel-specific parts as MlpSmem from CTL on, without the pair table.
-template <int NWG>
-struct NetSmem {
-    static constexpr uint32_t W0 = 0;
-    static constexpr uint32_t W1 = W0 + kNetW0;
-    static constexpr uint32_t W2 = W1 + kNetW12;
-    static constexpr uint32_t X = W2 + kNetW12;      // [NWG] tiles
-    static constexpr uint32_t H = X + NWG * kNetX;   // [NWG] tiles
-    static constexpr uint32_t W3 = H + NWG * kNetHt;
-    static constexpr uint32_t B3 = W3 + kNetHid * 4;
-    static constexpr uint32_t MBAR = B3 + 16;        // [NWG][2]
-    static constexpr uint32_t TSLOT = MBAR + 16 * NWG;
-    static constexpr uint32_t CTL = TSLOT + 4;
-    static constexpr uint32_t RED = (CTL + 4 + 15) / 16 * 16;
-    static constexpr uint32_t TINFO = RED + 64;
-    static constexpr uint32_t ACT = TINFO + kMlpChunk * kTinfo * 4;
-    static constexpr uint32_t GEO = ACT + kMlpChunk * 4;
-    static constexpr uint32_t END = (uint32_t)((GEO + sizeof(MlpGeo) + 127) / 128 * 128);
-    static_assert(X % 128 == 0 && H % 128 == 0 && W1 % 128 == 0 && W2 % 128 == 0, "tile alignment");
-    static_assert(MBAR % 8 == 0 && RED % 8 == 0, "alignment");
-};
-
-// The two site-energy networks the MLP kernels run: evaluator, layouts and
-// warpgroups of the sweep.
-struct NetSilu64 {  // MLP of mlp_tc.cuh: 20 -> 64 -> 64 -> 1, SiLU
-    using Eval = TcEval;
-    using Block = MlpBlock;
-    template <int NWG>
-    using Smem = MlpSmem<NWG>;
-    static constexpr int kSweepNWG = kSweepWG;
-    template <int NWG>
-    static __device__ TcLayout layout(uint32_t wg)
-    {
-        using M = MlpSmem<NWG>;
-        return TcLayout{M::X + wg * kTcX, M::H + wg * kTcH, M::W1, M::W2, M::B1, M::B2, M::W3, M::B3,
-                        M::MBAR + 16 * wg, M::TSLOT};
-    }
-};
-struct NetRelu96 {  // MLPNet of mlpnet_tc.cuh: 20 -> 96 -> 96 -> 96 -> 1, ReLU
-    using Eval = NetEval;
-    using Block = NetBlock;
-    template <int NWG>
-    using Smem = NetSmem<NWG>;
-    static constexpr int kSweepNWG = 2;  // the 28 KB hidden tiles of four would not fit
-    template <int NWG>
-    static __device__ NetLayout layout(uint32_t wg)
-    {
-        using M = NetSmem<NWG>;
-        return NetLayout{M::X + wg * kNetX, M::H + wg * kNetHt, M::W0, M::W1, M::W2, M::W3, M::B3, M::MBAR + 16 * wg,
-                         M::TSLOT};
-    }
-};
-
-// Site-energy models of the tensor-core sweep.
-constexpr int kModeMlp = 0, kModeMlpPair = 1;
-
-// The evaluator of this thread's warpgroup.
-template <class Net, int NWG>
-__device__ __forceinline__ typename Net::Eval mlp_evaluator(long long timeout_ns, int *status, int *abort_flag)
-{
-    const uint32_t wg = threadIdx.x >> 7;
-    typename Net::Eval E;
-    E.L = Net::template layout<NWG>(wg);
-    E.timeout_ns = timeout_ns;
-    E.status = status;
-    E.abort_flag = abort_flag;
-    E.tmem = 0;
-    E.phase1 = E.phase2 = 0;
-    E.bar = 1 + wg;
-    return E;
-}
-
-// Pair part of dE (pair + MLP models) from the packed post-swap neighbour
-// histograms of a (species B now) and b (species A now), 3 shells each; the
-// swapped partner is removed from shell 1.
-template <int NWG>
-__device__ __forceinline__ float pair_part(const SweepParams &P, const int *ha, const int *hb, int A, int B)
-{
-    const float *Dt = (const float *)(g_smem + MlpSmem<NWG>::D);
-    float dp = 0.f;
-    for (int m = 0; m < P.nshells; ++m) {
-        const float *D = Dt + ((m * kMaxSpecies + A) * kMaxSpecies + B) * kMaxSpecies;
-        for (int q = 0; q < P.S; ++q) {
-            float ca = (float)(((uint32_t)ha[m] >> (4 * q)) & 15u);
-            float cb = (float)(((uint32_t)hb[m] >> (4 * q)) & 15u);
-            if (m == 0) {
-                ca -= (q == A) ? 1.f : 0.f;
-                cb -= (q == B) ? 1.f : 0.f;
-            }
-            dp = fmaf(ca - cb, D[q], dp);
-        }
-    }
-    return dp;
-}
-
-// Copies the model (weights, pair table, geometry) and sets up the evaluators.
-template <class Net, int NWG>
-__device__ void mlp_cta_setup(typename Net::Eval &E, const void *W, const float *Dsrc, const MlpGeo *geo)
-{
-    using M = typename Net::template Smem<NWG>;
-    tc_load_weights((const typename Net::Block *)W, E.L);
-    const int tid = threadIdx.x, n = blockDim.x;
-    if constexpr (std::is_same<Net, NetSilu64>::value) {
-        if (Dsrc)
-            for (int i = tid; i < kDEntries; i += n) ((float *)(g_smem + M::D))[i] = Dsrc[i];
-    }
-    if (geo)
-        for (int i = tid; i < (int)(sizeof(MlpGeo) / 4); i += n) ((int *)(g_smem + M::GEO))[i] = ((const int *)geo)[i];
-    tc_setup(E, NWG);
-}
 
 // ---------------------------------------------------------------------------
 // Per-site energies of the whole lattice: e[i] = f(x_i), optionally stored
@@ -198,12 +37,12 @@ __device__ void mlp_cta_setup(typename Net::Eval &E, const void *W, const float 
 // warpgroup takes 128 consecutive sites per tile.
 // ---------------------------------------------------------------------------
 template <class Net>
-__global__ void __launch_bounds__(128 * kEvalWG) k_mlp_site_energy(const void *W, const int8_t *__restrict__ occ,
+__global__ void __launch_bounds__(128 * kStreamWG) k_mlp_site_energy(const void *W, const int8_t *__restrict__ occ,
                                                                    int nx, int ny, int nz, float *ecache,
                                                                    uint4 *fcache, double *part, long long timeout_ns,
                                                                    int *status, int *abort_flag)
 {
-    constexpr int NWG = kEvalWG;
+    constexpr int NWG = kStreamWG;
     using M = typename Net::template Smem<NWG>;
     typename Net::Eval E = mlp_evaluator<Net, NWG>(timeout_ns, status, abort_flag);
     mlp_cta_setup<Net, NWG>(E, W, nullptr, nullptr);
@@ -458,7 +297,7 @@ __device__ __forceinline__ void mlp_column(const SweepParams &P, const RepDesc &
                     const int base = (ti[15] + (tid >= 32 ? red_i[0] : 0)) * kOmega;
                     float dE = 0.f;
                     for (int e = 0; e < kOmega; ++e) dE += diff[base + e];
-                    if (HAS_PAIR) dE += pair_part<NWG>(P, ti + 8, ti + 11, A, B);
+                    if (HAS_PAIR) dE += pair_part((const float *)(g_smem + MlpSmem<NWG>::D), P.nshells, P.S, ti + 8, ti + 11, A, B);
                     const bool acc = metropolis<false>(dE, (uint32_t)ti[1], beta, nullptr, make_int2(0, 0));
                     ti[7] = acc ? 1 : 0;
                     if (acc) {
@@ -660,7 +499,7 @@ __global__ void __launch_bounds__(128 * kEvalWG) k_mlp_trace_eval(const __grid_c
             float dE = 0.f;
             for (int e = 0; e < kOmega; ++e) dE += fpost[tid * kOmega + e] - fpre[tid * kOmega + e];
             const int A = ti[3], B = ti[4];
-            if (HAS_PAIR && A != B) dE += pair_part<kEvalWG>(P, ti + 9, ti + 12, A, B);
+            if (HAS_PAIR && A != B) dE += pair_part((const float *)(g_smem + MlpSmem<kEvalWG>::D), P.nshells, P.S, ti + 9, ti + 12, A, B);
             const bool acc = metropolis<false>(dE, (uint32_t)ti[2], P.temp.beta[0], nullptr, make_int2(0, 0));
             if (dE_out) dE_out[c] = dE;
             if (acc_out) acc_out[c] = acc ? 1 : 0;
@@ -840,6 +679,8 @@ int shell_between(int sa, const Cell &a, int sb, const Cell &b)
     return d2 == 3 ? 1 : (d2 == 4 ? 2 : (d2 == 8 ? 3 : 0));
 }
 
+}  // namespace
+
 // Omega of every (trial sublattice, partner direction) with the shells in
 // which each zone site sees a and b; fails on a geometry inconsistency.
 bool build_mlp_geo(MlpGeo &G)
@@ -882,6 +723,8 @@ bool build_mlp_geo(MlpGeo &G)
     return true;
 }
 
+namespace {
+
 bool mlp_shape_ok(const smc_lattice *lat)
 {
     return lc_edge(lat->nx) == 4 && lc_edge(lat->ny) == 4 && lc_edge(lat->nz) == 4;
@@ -920,8 +763,10 @@ void make_net_block(const smc_model *m, NetBlock &W)
     W.b3 = m->net_b3;
 }
 
+}  // namespace
+
 // Copies the model's weight block (MlpBlock or NetBlock) to dst (device).
-smc_status copy_weights(const smc_model *m, void *dst, cudaStream_t stream)
+smc_status mlp_copy_weights(const smc_model *m, void *dst, cudaStream_t stream)
 {
     static MlpBlock Wm;
     static NetBlock Wn;
@@ -940,10 +785,6 @@ smc_status copy_weights(const smc_model *m, void *dst, cudaStream_t stream)
     return e == cudaSuccess ? SMC_OK : cuda_fail(e, "cudaMemcpyAsync(network weights)");
 }
 
-constexpr size_t kWeightBytes = sizeof(MlpBlock) > sizeof(NetBlock) ? sizeof(MlpBlock) : sizeof(NetBlock);
-
-}  // namespace
-
 // E (+)= sum_i f(x_i); writes the per-site energies to ecache and the
 // features to fcache when non-NULL.
 // W is the device weight block of Net; part needs room for kTcMaxCtasPerSm CTAs per SM;
@@ -953,23 +794,14 @@ static smc_status mlp_energy_launch(Workspace *ws, const smc_lattice *lat, const
                                     float *ecache, uint4 *fcache, double *part, int *abort_flag, double *e,
                                     int accumulate, cudaStream_t stream)
 {
-    const size_t smem = Net::template Smem<kEvalWG>::END;
+    const size_t smem = Net::template Smem<kStreamWG>::END;
     auto kern = k_mlp_site_energy<Net>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return cuda_fail(err, "cudaFuncSetAttribute(k_mlp_site_energy)");
-    int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128 * kEvalWG, smem);
-    if (err != cudaSuccess) return cuda_fail(err, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-    if (per_sm > kTcMaxCtasPerSm) {
-        // more resident CTAs than tensor-memory allocations: a CTA would wait in tcgen05.alloc
-        set_error("internal error: MLP energy kernel occupancy exceeds tensor memory");
-        return SMC_ERR_STATE;
-    }
-    per_sm = std::max(1, per_sm);
     const long long N = 2LL * lat->nx * lat->ny * lat->nz;
     const long long tiles = (N + kTcRows - 1) / kTcRows;
-    const int grid = (int)std::max(1LL, std::min<long long>((long long)per_sm * ws->num_sms, tiles));
-    kern<<<grid, 128 * kEvalWG, smem, stream>>>(W, occ, lat->nx, lat->ny, lat->nz, ecache, fcache, part,
+    const int grid = (int)std::max(1LL, std::min<long long>(ws->num_sms, tiles));
+    kern<<<grid, 128 * kStreamWG, smem, stream>>>(W, occ, lat->nx, lat->ny, lat->nz, ecache, fcache, part,
                                                            debug_timeout_ns(), ws->status, abort_flag);
     err = cudaGetLastError();
     if (err != cudaSuccess) return cuda_fail(err, "k_mlp_site_energy");
@@ -994,7 +826,7 @@ smc_status launch_mlp_energy(const smc_lattice *lat, const smc_model *m, const i
     const size_t need = off_part + sizeof(double) * kTcMaxCtasPerSm * (size_t)std::max(ws->num_sms, 1);
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, need, &st);
     if (!scr) return st;
-    st = copy_weights(m, scr + off_w, stream);
+    st = mlp_copy_weights(m, scr + off_w, stream);
     if (st != SMC_OK) return st;
     cudaError_t err = cudaMemsetAsync(scr + off_abort, 0, 16, stream);
     if (err != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync(abort word)");
@@ -1123,6 +955,14 @@ smc_status launch_mlp_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     d.rep = replica;
     d.vec = (d.nx % 16 == 0) && ((uintptr_t)occ % 16 == 0);
     if (has_pair) fill_pair_D(m, P.S, P);
+    // A call whose trials evaluate more rows than there are feature vectors
+    // evaluates each vector once and looks the others up.
+    if (mlp_table_wanted(lat, nsweeps)) {
+        bool taken = false;
+        st = launch_mlp_table_sweep(lat, m, occ, seed, replica, sweep0, nsweeps, kT, e_acc, n_acc, P.D.df, &taken,
+                                    stream);
+        if (st != SMC_OK || taken) return st;
+    }
 
     // workspace: [flags | part_e | part_n | ticket, abort | weights | energy parts | E cache | F cache]
     const size_t nt = (size_t)P.ntiles;
@@ -1144,7 +984,7 @@ smc_status launch_mlp_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     P.mlpw = scr + off_w;
     P.ecache = (float *)(scr + off_cache);
     P.fcache = (uint4 *)(scr + off_fcache);
-    st = copy_weights(m, scr + off_w, stream);
+    st = mlp_copy_weights(m, scr + off_w, stream);
     if (st != SMC_OK) return st;
     cudaError_t e = cudaMemsetAsync(scr, 0, off_misc + 16, stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(sweep scratch)");
@@ -1220,7 +1060,7 @@ smc_status launch_mlp_trace(const smc_lattice *lat, const smc_model *m, int8_t *
     int *swap_a = (int *)scr, *swap_b = swap_a + ntr;
     P.abort_flag = (int *)(scr + off_abort);
     P.mlpw = scr + off_w;
-    st = copy_weights(m, scr + off_w, stream);
+    st = mlp_copy_weights(m, scr + off_w, stream);
     if (st != SMC_OK) return st;
     cudaError_t e = cudaMemsetAsync(scr + off_abort, 0, 16, stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(abort word)");
