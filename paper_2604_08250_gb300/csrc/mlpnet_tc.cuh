@@ -147,6 +147,15 @@ __device__ __forceinline__ void tc_timeout(NetEval &E)
     atomicExch(E.abort_flag, 1);
 }
 
+// BF16 pair of relu(lo), relu(hi): the maximum is taken after rounding (the
+// same value: rounding keeps sign and order, and a NaN gives 0 either way), one
+// packed instruction instead of two.
+__device__ __forceinline__ uint32_t pack_relu(float lo, float hi)
+{
+    const __nv_bfloat162 v = __hmax2(__floats2bfloat162_rn(lo, hi), __float2bfloat162_rn(0.f));
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+
 // relu of this warp's 32 rows x 96 columns of D, as BF16, into the H tile.
 __device__ __forceinline__ void net_epilogue(NetEval &E, uint32_t r, uint32_t lane_base)
 {
@@ -160,8 +169,7 @@ __device__ __forceinline__ void net_epilogue(NetEval &E, uint32_t r, uint32_t la
             uint32_t w[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                w[u] = pack_bf16(fmaxf(__uint_as_float(v[8 * kc + 2 * u]), 0.f),
-                                 fmaxf(__uint_as_float(v[8 * kc + 2 * u + 1]), 0.f));
+                w[u] = pack_relu(__uint_as_float(v[8 * kc + 2 * u]), __uint_as_float(v[8 * kc + 2 * u + 1]));
             *(uint4 *)(g_smem + E.L.h + tn_off112(r, 4 * third + kc)) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
