@@ -12,15 +12,21 @@
 // shell, w = Philox4x32-10(key seed, counter (s, replica, sweep lo, hi)),
 // Metropolis on r = w0 & (2^29 - 1) as for the BCC lattice.
 //
-// One thread per trial and one launch per mini-step: the trials of a
-// mini-step touch disjoint read and write sets (pinned exhaustively on the
-// CPU for 1-3 shells), and consecutive launches are ordered by the stream.
+// One thread per trial.  Rows of up to 1024 cells run the four mini-steps of a
+// group in one launch on rows in shared memory (k_fcc_group here,
+// k_qsro_group in qsro_group.cuh; 256^3 cells, 2 shells: 41 us per group of
+// the pair model and 92 of the qSRO model, against 91 and 188 with a launch
+// per mini-step; 128^3: 13 and 22 against 66 and 104).  Longer rows run one
+// launch per mini-step (k_fcc_ministep, k_fcc_qsro_ministep, described next):
+// the trials of a mini-step touch disjoint read and write sets (pinned
+// exhaustively on the CPU for 1-3 shells), and consecutive launches are
+// ordered by the stream.
 // dE sums the changed bonds: with every axis at least 8 cells no shell
 // aliases, so a's neighbours other than b and b's other than a each flip
 // one bond, dE = sum_j D_m(q_j) over a's zone - sum_j D_m(q_j) over b's,
-// D_m(q) = V_m(B, q) - V_m(A, q).  The same kernel records the trace (dE,
-// decision) of a mini-step, so a sweep equals its traced mini-steps bit for
-// bit.
+// D_m(q) = V_m(B, q) - V_m(A, q).  The kernel of the sweep records the trace
+// (dE, decision) of a mini-step, so a sweep equals its traced mini-steps bit
+// for bit.
 //
 // Link cells away from the box faces (1 <= c < NL-1 on every axis) reach
 // every neighbour of a and b without a periodic wrap: a neighbour is the
@@ -42,7 +48,7 @@
 #include <type_traits>
 #include <vector>
 
-#include "sweep_common.cuh"
+#include "qsro_group.cuh"
 
 namespace smc {
 
@@ -263,6 +269,110 @@ __global__ void __launch_bounds__(256) k_fcc_ministep(const __grid_constant__ Fc
     }
     if (P.dE_out) P.dE_out[c] = (float)dw;
     if (P.acc_out) P.acc_out[c] = acc ? 1 : 0;
+}
+
+// The same trials, one launch per group of four mini-steps (row_group.cuh):
+// species come from the column's rows in shared memory, a neighbour of a at
+// offA[t] and one of b at offB[t][dir] bytes from a.  Sums in the order of
+// k_fcc_ministep.
+constexpr int kFgB = kMaxShells * 512, kFgWords = kFgB + 4 * 44 * 16;  // tables: D rows, per sublattice offB
+
+struct FccGroup {
+    RowGroup G;
+    uint64_t seed, sweep;
+    uint32_t replica;
+    float beta;
+    int2 tinfo;
+    const uint32_t *tab;
+    const uint32_t *tables;  // D rows, then per sublattice [44][16]: offB (42), b's own offset and its dx
+    int8_t *occ;
+    double *part_e;
+    long long *part_n;
+    float *dE_out;
+    uint8_t *acc_out;
+    int offA[42];
+};
+
+template <bool IS_INT, int NSH>
+__global__ void __launch_bounds__(kRgThreads) k_fcc_group(const __grid_constant__ FccGroup P)
+{
+    using T = typename Acc<IS_INT>::T;
+    using Word = typename std::conditional<IS_INT, int, float>::type;
+    using Wide = typename std::conditional<IS_INT, long long, float>::type;  // as k_fcc_ministep
+    constexpr int NV = NSH == 1 ? 12 : (NSH == 2 ? 18 : 42);
+    const RowGroup &G = P.G;
+    const Word *sT = (const Word *)g_smem;          // [NSH][64][8]
+    const int *sB = (const int *)(sT + NSH * 512);  // [44][16]
+    constexpr uint32_t rows0 = (uint32_t)(NSH * 512 + 44 * 16) * 4;
+    const int tid = threadIdx.x, c = tid / G.tpc, tt = tid - c * G.tpc, col = blockIdx.x * G.C + c;
+    const bool on = col < G.ncol;
+    const int y0 = 4 * (col % G.NLy) + G.dy, z0 = 4 * (col / G.NLy) + G.dz;
+    int *rown = (int *)(g_smem + rows0 + c * kRgRowBytes);
+    const uint32_t base = rows0 + G.C * kRgRowBytes + (uint32_t)(c * G.rows.n * G.pitch);
+    if (on) rg_rows(G, rown, y0, z0, tt);
+    __syncthreads();
+    if (on) rg_stage<1>(G, (const unsigned char *)P.occ, base, G.pitch, G.unit, G.inv, rown, tt);
+    for (int i = tid; i < NSH * 512; i += blockDim.x) ((uint32_t *)g_smem)[i] = __ldg(P.tables + i);
+    for (int i = tid; i < 44 * 16; i += blockDim.x)
+        ((uint32_t *)g_smem)[NSH * 512 + i] = __ldg(P.tables + kFgB + G.sub * 44 * 16 + i);
+    const bool active = on && tt < G.NLx;
+    const int lc = col * G.NLx + tt;
+    double accE = 0.0;
+    long long accN = 0;
+    rg_wait();
+    for (int dx = G.dx0; dx < G.dx1; ++dx) {
+        if (active) {
+            const int x = 4 * tt + dx;
+            const uint32_t a = (uint32_t)(((G.sub * G.nz + z0) * G.ny + y0) * G.nx + x);
+            const U4 w = philox10(U4{a, P.replica, (uint32_t)P.sweep, (uint32_t)(P.sweep >> 32)}, (uint32_t)P.seed,
+                                  (uint32_t)(P.seed >> 32));
+            const uint32_t r = w.x & kRMask;
+            const int dir = (int)(((uint64_t)w.y * 12u) >> 32), opp = 11 - dir;
+            const uint32_t at = base + kRgBody + x;
+            const int *ob = sB + dir;
+            const uint32_t bt = at + ob[42 * 16];
+            uint32_t qa[NV], qb[NV];
+#pragma unroll
+            for (int t = 0; t < NV; ++t) qa[t] = SM8(at + P.offA[t]);
+#pragma unroll
+            for (int t = 0; t < NV; ++t) qb[t] = SM8(at + ob[t * 16]);
+            const int A = SM8(at) & 7, B = SM8(bt) & 7;
+            const Word *row = sT + (A * 8 + B) * 8;
+            Wide dw = Wide(0);
+#pragma unroll
+            for (int t = 0; t < NV; ++t) {
+                const Word v = row[fcc_shell_off(t) + (qa[t] & 7)];
+                if (t >= 12 || t != dir) dw += (Wide)v;
+            }
+#pragma unroll
+            for (int t = 0; t < NV; ++t) {
+                const Word v = row[fcc_shell_off(t) + (qb[t] & 7)];
+                if (t >= 12 || t != opp) dw -= (Wide)v;
+            }
+            // a dE beyond the int range is rejected anyway (the acceptance table is shorter)
+            T dE;
+            if constexpr (IS_INT)
+                dE = (T)(dw > 0x7FFFFFFFLL ? 0x7FFFFFFFLL : (dw < -0x7FFFFFFFLL ? -0x7FFFFFFFLL : dw));
+            else
+                dE = dw;
+            const bool acc = metropolis<IS_INT>(dE, r, P.beta, P.tab, P.tinfo);
+            if (acc) {
+                rg_put<int8_t>(at, x, G.nx, (int8_t)B);
+                rg_put<int8_t>(bt, x + ob[43 * 16], G.nx, (int8_t)A);
+                accE += (double)dw;
+                ++accN;
+            }
+            if (P.dE_out) P.dE_out[lc] = (float)dw;
+            if (P.acc_out) P.acc_out[lc] = acc ? 1 : 0;
+        }
+        __syncthreads();
+    }
+    if (on)
+        rg_store<1>(G, (unsigned char *)P.occ, base, G.pitch, G.unit, G.inv, G.rows.nwr, rown, tt);
+    if (active && accN) {
+        P.part_e[lc] += accE;
+        P.part_n[lc] += accN;
+    }
 }
 
 __device__ __forceinline__ int3 fcc_woff(int w) { return make_int3(w % 7 - 3, (w / 7) % 7 - 3, w / 49 - 3); }
@@ -701,6 +811,131 @@ smc_status fcc_sweep_tables(const smc_lattice *lat, const smc_model *m, std::vec
     return SMC_OK;
 }
 
+// Half-unit basis of sublattice s, and the sublattice of a half-unit parity.
+std::array<int, 3> fcc_basis(int s) { return {(s == 1 || s == 2) ? 1 : 0, (s == 1 || s == 3) ? 1 : 0, (s == 2 || s == 3) ? 1 : 0}; }
+
+int floor_half(int v) { return v >= 0 ? v / 2 : -((1 - v) / 2); }
+
+// The shell vectors in table order (shell 1: 0-11, 2: 12-17, 3: 18-41).
+std::vector<std::array<int, 3>> fcc_vectors()
+{
+    std::vector<std::array<int, 3>> vec;
+    for (int sh = 1; sh <= 3; ++sh)
+        for (int x = -2; x <= 2; ++x)
+            for (int y = -2; y <= 2; ++y)
+                for (int z = -2; z <= 2; ++z)
+                    if (x * x + y * y + z * z == 2 * sh && ((x + y + z) & 1) == 0) vec.push_back({x, y, z});
+    return vec;
+}
+
+// Rows that the trials of sublattice `sub` reach with nv vectors around a and
+// b: the row of a, the rows of its first-shell sites, the others.  slot[y+3][z+3]:
+// row of a half-unit offset (-1: none).  Returns false on an inconsistency.
+int fcc_rows(int nsh) { return nsh == 1 ? 25 : (nsh == 2 ? 37 : 45); }
+bool fcc_rowset(int sub, int nv, RowSet &R, int slot[7][7])
+{
+    const std::vector<std::array<int, 3>> vec = fcc_vectors();
+    const std::array<int, 3> b = fcc_basis(sub);
+    memset(&R, 0, sizeof R);
+    for (int i = 0; i < 7; ++i)
+        for (int j = 0; j < 7; ++j) slot[i][j] = -1;
+    auto need = [&](int hy, int hz) {
+        if (slot[hy + 3][hz + 3] >= 0) return;
+        const int px = (hy + hz) & 1;  // half-unit offsets of a site sum to an even number
+        const int par = (((b[0] + px) & 1) << 2) | (((b[1] + hy) & 1) << 1) | ((b[2] + hz) & 1);
+        slot[hy + 3][hz + 3] = R.n;
+        R.sub[R.n] = (signed char)(par == 0 ? 0 : (par == 6 ? 1 : (par == 5 ? 2 : 3)));
+        R.dy[R.n] = (signed char)floor_half(b[1] + hy);
+        R.dz[R.n] = (signed char)floor_half(b[2] + hz);
+        ++R.n;
+    };
+    need(0, 0);
+    for (int d = 0; d < 12; ++d) need(vec[d][1], vec[d][2]);
+    R.nwr = R.n;
+    for (int t = 0; t < nv; ++t) need(vec[t][1], vec[t][2]);
+    for (int d = 0; d < 12; ++d)
+        for (int t = 0; t < nv; ++t) need(vec[d][1] + vec[t][1], vec[d][2] + vec[t][2]);
+    return R.nwr == 9 && R.n == fcc_rows(nv == 12 ? 1 : (nv == 18 ? 2 : 3)) && R.sub[0] == sub && R.dy[0] == 0 && R.dz[0] == 0;
+}
+
+// Byte offset from a (es-byte cells, rows `pitch` apart) of half-unit vector v.
+int fcc_group_off(int sub, const int slot[7][7], int pitch, int es, int vx, int vy, int vz)
+{
+    return slot[vy + 3][vz + 3] * pitch + es * floor_half(fcc_basis(sub)[0] + vx);
+}
+
+// Per-sublattice offsets of k_fcc_group, appended to the D rows in w.
+bool fcc_group_tables(int nsh, int pitch, std::vector<uint32_t> &w, RowSet rows[4], int offA[4][42])
+{
+    const std::vector<std::array<int, 3>> vec = fcc_vectors();
+    const int nv = nsh == 1 ? 12 : (nsh == 2 ? 18 : 42);
+    w.resize(kFgWords, 0u);
+    for (int s = 0; s < 4; ++s) {
+        int slot[7][7];
+        if (!fcc_rowset(s, nv, rows[s], slot)) return false;
+        uint32_t *o = &w[(size_t)(kFgB + s * 44 * 16)];
+        for (int t = 0; t < 42; ++t) offA[s][t] = 0;
+        for (int t = 0; t < nv; ++t) {
+            offA[s][t] = fcc_group_off(s, slot, pitch, 1, vec[t][0], vec[t][1], vec[t][2]);
+            for (int d = 0; d < 12; ++d)
+                o[t * 16 + d] = (uint32_t)fcc_group_off(s, slot, pitch, 1, vec[d][0] + vec[t][0], vec[d][1] + vec[t][1],
+                                                        vec[d][2] + vec[t][2]);
+        }
+        for (int d = 0; d < 12; ++d) {
+            o[42 * 16 + d] = (uint32_t)fcc_group_off(s, slot, pitch, 1, vec[d][0], vec[d][1], vec[d][2]);
+            o[43 * 16 + d] = (uint32_t)floor_half(fcc_basis(s)[0] + vec[d][0]);
+        }
+    }
+    return true;
+}
+
+// The FCC lattice for k_qsro_group.
+struct FccQsro {
+    struct Words {};
+    static __host__ __device__ constexpr int zone(int nsh) { return nsh == 1 ? 18 : (nsh == 2 ? 26 : 58); }
+    static __host__ __device__ constexpr int code(int nsh, int e) { return fcc_zone_code(nsh, e); }
+    static __host__ __device__ constexpr int qoff(int m) { return fcc_qoff(m); }
+    static __host__ __device__ constexpr int qmask(int m) { return fcc_qmask(m); }
+    static __device__ __forceinline__ Words words(const QsroGroup &, int) { return Words{}; }
+    static __device__ __forceinline__ void draw(const QsroGroup &P, const Words &, int site, int, uint32_t &r, int &dir)
+    {
+        const U4 w = philox10(U4{(uint32_t)site, P.replica, (uint32_t)P.sweep, (uint32_t)(P.sweep >> 32)},
+                              (uint32_t)P.seed, (uint32_t)(P.seed >> 32));
+        r = w.x & kRMask;
+        dir = (int)(((uint64_t)w.y * 12u) >> 32);
+    }
+};
+
+// The table of k_qsro_group from the zone lists of fcc_qsro_tables in w.
+bool fcc_qsro_group_tables(int nsh, int pitch, const std::vector<uint32_t> &w, std::vector<uint32_t> &out, RowSet rows[4])
+{
+    out.assign((size_t)qg_words(4), 0u);
+    memcpy(out.data(), w.data(), (size_t)(kMaxShells * 520) * 4);
+    const int nz = FccQsro::zone(nsh), nv = nsh == 1 ? 12 : (nsh == 2 ? 18 : 42);
+    for (int s = 0; s < 4; ++s) {
+        int slot[7][7];
+        if (!fcc_rowset(s, nv, rows[s], slot)) return false;
+        for (int d = 0; d < 12; ++d)
+            for (int e = 0; e <= nz; ++e) {
+                const int o = (int)(e < nz ? w[(size_t)(kQZ + d * kQZmax + e)] : w[(size_t)(kQV1 + d)]);
+                const int hx = o % 7 - 3, hy = (o / 7) % 7 - 3, hz = o / 49 - 3;
+                const int sl = slot[hy + 3][hz + 3];
+                if (sl < 0) return false;
+                out[(size_t)(kQgOff + s * kQgSub + (e < nz ? e : kQgZone) * kQgDirs + d)] =
+                    qg_pack(sl, pitch, floor_half(fcc_basis(s)[0] + hx));
+            }
+    }
+    return true;
+}
+
+using FccGroupKernel = void (*)(FccGroup);
+
+template <bool IS_INT>
+FccGroupKernel pick_fcc_group(int nshells)
+{
+    return nshells == 1 ? k_fcc_group<IS_INT, 1> : (nshells == 2 ? k_fcc_group<IS_INT, 2> : k_fcc_group<IS_INT, 3>);
+}
+
 using FccKernel = void (*)(FccStep, int);
 
 template <bool IS_INT>
@@ -749,6 +984,32 @@ smc_status launch_fcc_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     std::vector<uint32_t> words;
     st = is_qsro ? fcc_qsro_tables(lat, m, words) : fcc_sweep_tables(lat, m, words);
     if (st != SMC_OK) return st;
+    // Rows of up to 1024 cells run a group of mini-steps per launch.
+    static FccGroup gp;
+    RowSet grows[4];
+    int goff[4][42];
+    bool grouped = false;
+    const size_t fixed = (size_t)(m->nshells * 512 + 44 * 16) * 4;
+    if (!is_qsro && rg_plan(lat, occ, ws->num_sms, ws->smem_optin, fixed, fcc_rows(m->nshells), 0, gp.G)) {
+        words.resize(kFgB);
+        if (!fcc_group_tables(m->nshells, gp.G.pitch, words, grows, goff)) {
+            set_error("internal error: FCC row table");
+            return SMC_ERR_STATE;
+        }
+        grouped = true;
+    }
+    static QsroGroup gq;
+    const size_t qfixed = qg_fixed(m->nshells, FccQsro::zone(m->nshells));
+    const bool qgrouped =
+        is_qsro && rg_plan(lat, occ, ws->num_sms, ws->smem_optin, qfixed, fcc_rows(m->nshells), m->nshells == 3 ? 2 : 1, gq.G);
+    if (qgrouped) {
+        std::vector<uint32_t> gwords;
+        if (!fcc_qsro_group_tables(m->nshells, gq.G.pitch, words, gwords, grows)) {
+            set_error("internal error: FCC row table");
+            return SMC_ERR_STATE;
+        }
+        words.swap(gwords);
+    }
     // workspace: [part_e | part_n | ministep tables | acceptance tables | reduction scratch | qSRO count cache]
     const size_t off_pn = (size_t)nc * 8, off_w = off_pn + (size_t)nc * 8, off_tab = off_w + words.size() * 4;
     const size_t off_red = (off_tab + tabs.size() * 4 + 255) / 256 * 256, off_q = off_red + lc_reduce_bytes();
@@ -768,6 +1029,43 @@ smc_status launch_fcc_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     P.tab = (const uint32_t *)(scr + off_tab);
     P.part_e = (double *)scr;
     P.part_n = (long long *)(scr + off_pn);
+    if (grouped) {
+        const FccGroupKernel kern = is_int ? pick_fcc_group<true>(m->nshells) : pick_fcc_group<false>(m->nshells);
+        const size_t smem = fixed + (size_t)gp.G.C * (kRgRowBytes + (size_t)grows[0].n * gp.G.pitch);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_fcc_group)");
+        gp.seed = seed;
+        gp.replica = replica;
+        gp.tab = P.tab;
+        gp.tables = P.tables;
+        gp.occ = occ;
+        gp.part_e = P.part_e;
+        gp.part_n = P.part_n;
+        gp.dE_out = trace_dE;
+        gp.acc_out = trace_acc;
+        const int blocks = (gp.G.ncol + gp.G.C - 1) / gp.G.C;
+        for (int t = 0; t < nsweeps; ++t) {
+            gp.sweep = sweep0 + (uint64_t)t;
+            gp.beta = (float)(1.0 / kT[t]);
+            gp.tinfo = tinfo[t];
+            const int g0 = trace_k >= 0 ? trace_k >> 2 : 0, g1 = trace_k >= 0 ? g0 + 1 : 64;
+            gp.G.dx0 = trace_k >= 0 ? trace_k & 3 : 0;
+            gp.G.dx1 = trace_k >= 0 ? gp.G.dx0 + 1 : 4;
+            for (int g = g0; g < g1; ++g) {
+                gp.G.dy = g & 3;
+                gp.G.dz = (g >> 2) & 3;
+                gp.G.sub = g >> 4;
+                gp.G.rows = grows[gp.G.sub];
+                memcpy(gp.offA, goff[gp.G.sub], sizeof gp.offA);
+                kern<<<blocks, gp.G.C * gp.G.tpc, smem, stream>>>(gp);
+            }
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return cuda_fail(e, "k_fcc_group");
+        }
+        if (e_acc || n_acc)
+            return launch_lc_reduce(P.part_e, P.part_n, nc, scr + off_red, e_acc, (long long *)n_acc, stream);
+        return SMC_OK;
+    }
     const int threads = 256;
     P.n_int = (P.NLx > 2 && P.NLy > 2 && P.NLz > 2) ? (P.NLx - 2) * (P.NLy - 2) * (P.NLz - 2) : 0;
     P.n_bnd = nc - P.n_int;
@@ -782,6 +1080,23 @@ smc_status launch_fcc_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
         k_fcc_qsro_cache<<<cb, 256, 0, stream>>>(static_cast<const FccStep &>(P));
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "k_fcc_qsro_cache");
+    }
+    if (qgrouped) {
+        gq.seed = seed;
+        gq.replica = replica;
+        gq.tables = P.tables;
+        gq.occ = occ;
+        gq.qcache = P.qcache;
+        gq.part_e = P.part_e;
+        gq.part_n = P.part_n;
+        gq.dE_out = trace_dE;
+        gq.acc_out = trace_acc;
+        const size_t smem = qfixed + (size_t)gq.G.C * (kRgRowBytes + (size_t)grows[0].n * (gq.G.pitch + gq.G.pitchq));
+        auto gk = m->nshells == 1 ? k_qsro_group<FccQsro, 1>
+                                  : (m->nshells == 2 ? k_qsro_group<FccQsro, 2> : k_qsro_group<FccQsro, 3>);
+        st = qg_launch(gk, gq, grows, smem, sweep0, nsweeps, kT, 64, trace_k, stream);
+        if (st != SMC_OK || (!e_acc && !n_acc)) return st;
+        return launch_lc_reduce(P.part_e, P.part_n, nc, scr + off_red, e_acc, (long long *)n_acc, stream);
     }
     for (int t = 0; t < nsweeps; ++t) {
         P.sweep = sweep0 + (uint64_t)t;

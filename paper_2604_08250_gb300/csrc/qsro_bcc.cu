@@ -1,7 +1,10 @@
 // qsro_bcc.cu -- qSRO sweeps on the BCC lattice (Sec. IV-B, Eq.
 // quadratic_local_SRO; Algorithm 1 with 4x4x4 link cells, 128 mini-steps):
-// one thread per trial and one launch per mini-step, the trials of a
-// mini-step being independent (read/write sets pinned on the CPU).
+// one thread per trial, the trials of a mini-step being independent
+// (read/write sets pinned on the CPU).  Rows of up to 1024 cells run the four
+// mini-steps of a group in one launch on rows in shared memory
+// (qsro_group.cuh; 256^3, 2 shells: 65 us per group against 139 with a launch
+// per mini-step), longer ones k_bq_ministep, a launch per mini-step.
 //
 // Site j's energy changes only through the species of its neighbours a and
 // b: with a in shell ma of j and b in shell mb (0 = neither),
@@ -28,7 +31,7 @@
 #include <type_traits>
 #include <vector>
 
-#include "sweep_common.cuh"
+#include "qsro_group.cuh"
 
 namespace smc {
 
@@ -432,6 +435,72 @@ smc_status bq_tables(const smc_lattice *lat, const smc_model *m, std::vector<uin
     return SMC_OK;
 }
 
+// The BCC lattice for k_qsro_group.
+struct BccQsro {
+    using Words = U4;  // the four trial sites of a link cell's row share one Philox block
+    static __host__ __device__ constexpr int zone(int nsh) { return nsh == 1 ? 14 : (nsh == 2 ? 20 : 38); }
+    static __host__ __device__ constexpr int code(int nsh, int e) { return bq_code(nsh, e); }
+    static __host__ __device__ constexpr int qoff(int m) { return bq_qoff(m); }
+    static __host__ __device__ constexpr int qmask(int m) { return bq_qmask(m); }
+    static __device__ __forceinline__ Words words(const QsroGroup &P, int site)
+    {
+        return philox10(U4{(uint32_t)site >> 2, P.replica, (uint32_t)P.sweep, (uint32_t)(P.sweep >> 32)},
+                        (uint32_t)P.seed, (uint32_t)(P.seed >> 32));
+    }
+    static __device__ __forceinline__ void draw(const QsroGroup &, const Words &w, int, int dx, uint32_t &r, int &dir)
+    {
+        const uint32_t word = pick_word(w, (uint32_t)dx);
+        r = word & kRMask;
+        dir = (int)(word >> kRBits);
+    }
+};
+
+int bq_floor_half(int v) { return v >= 0 ? v / 2 : -((1 - v) / 2); }
+
+int bq_rows(int nsh) { return nsh == 1 ? 13 : (nsh == 2 ? 21 : 25); }
+
+// Rows that the trials of sublattice `sub` reach (row_group.cuh: the row of a,
+// the rows of its first-shell sites, the others) and the table of k_qsro_group,
+// from the zone lists of bq_tables in w.
+bool bq_group_tables(int nsh, int pitch, const std::vector<uint32_t> &w, std::vector<uint32_t> &out, RowSet rows[2])
+{
+    out.assign((size_t)qg_words(2), 0u);
+    memcpy(out.data(), w.data(), (size_t)(kMaxShells * 520) * 4);
+    const int nz = BccQsro::zone(nsh);
+    for (int s = 0; s < 2; ++s) {
+        RowSet &R = rows[s];
+        memset(&R, 0, sizeof R);
+        int slot[7][7];
+        for (auto &v : slot)
+            for (int &x : v) x = -1;
+        auto need = [&](int hy, int hz) {
+            if (((hy ^ hz) & 1) || slot[hy + 3][hz + 3] >= 0) return;
+            slot[hy + 3][hz + 3] = R.n;
+            R.sub[R.n] = (signed char)((s + hy) & 1);
+            R.dy[R.n] = (signed char)bq_floor_half(s + hy);
+            R.dz[R.n] = (signed char)bq_floor_half(s + hz);
+            ++R.n;
+        };
+        need(0, 0);
+        for (int y = -1; y <= 1; y += 2)
+            for (int z = -1; z <= 1; z += 2) need(y, z);
+        R.nwr = R.n;
+        for (int pass = 0; pass < 2; ++pass)
+            for (int d = 0; d < 8; ++d)
+                for (int e = 0; e <= nz; ++e) {
+                    const int o = (int)(e < nz ? w[(size_t)(kBqZ + d * kBqZmax + e)] : w[(size_t)(kBqV1 + d)]);
+                    const int hx = o % 7 - 3, hy = (o / 7) % 7 - 3, hz = o / 49 - 3;
+                    need(hy, hz);
+                    const int sl = slot[hy + 3][hz + 3];
+                    if (sl < 0) return false;
+                    out[(size_t)(kQgOff + s * kQgSub + (e < nz ? e : kQgZone) * kQgDirs + d)] =
+                        qg_pack(sl, pitch, bq_floor_half(s + hx));
+                }
+        if (R.nwr != 5 || R.n != bq_rows(nsh) || R.sub[0] != s) return false;
+    }
+    return true;
+}
+
 using BqKernel = void (*)(BqStep, int);
 
 }  // namespace
@@ -486,6 +555,20 @@ smc_status launch_qsro_ministeps(const smc_lattice *lat, const smc_model *m, int
     std::vector<uint32_t> words;
     st = bq_tables(lat, m, words);
     if (st != SMC_OK) return st;
+    // Rows of up to 1024 cells run a group of mini-steps per launch.
+    static QsroGroup gp;
+    RowSet rows[2];
+    std::vector<uint32_t> gwords;
+    const size_t fixed = qg_fixed(m->nshells, BccQsro::zone(m->nshells));
+    const bool grouped = rg_plan(lat, occ, ws->num_sms, ws->smem_optin, fixed, bq_rows(m->nshells),
+                                 m->nshells == 3 ? 2 : 1, gp.G);
+    if (grouped) {
+        if (!bq_group_tables(m->nshells, gp.G.pitch, words, gwords, rows)) {
+            set_error("internal error: BCC qSRO row table");
+            return SMC_ERR_STATE;
+        }
+        words.swap(gwords);
+    }
     // workspace: [part_e | part_n | tables | reduction scratch | count cache]
     const size_t off_pn = (size_t)nc * 8, off_w = off_pn + (size_t)nc * 8;
     const size_t off_red = (off_w + words.size() * 4 + 255) / 256 * 256, off_q = off_red + lc_reduce_bytes();
@@ -511,6 +594,23 @@ smc_status launch_qsro_ministeps(const smc_lattice *lat, const smc_model *m, int
     k_bq_cache<<<cb, 256, 0, stream>>>(P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "k_bq_cache");
+    if (grouped) {
+        gp.seed = seed;
+        gp.replica = replica;
+        gp.tables = P.tables;
+        gp.occ = occ;
+        gp.qcache = P.qcache;
+        gp.part_e = P.part_e;
+        gp.part_n = P.part_n;
+        gp.dE_out = trace_dE;
+        gp.acc_out = trace_acc;
+        const size_t smem = fixed + (size_t)gp.G.C * (kRgRowBytes + (size_t)rows[0].n * (gp.G.pitch + gp.G.pitchq));
+        auto gk = m->nshells == 1 ? k_qsro_group<BccQsro, 1>
+                                  : (m->nshells == 2 ? k_qsro_group<BccQsro, 2> : k_qsro_group<BccQsro, 3>);
+        st = qg_launch(gk, gp, rows, smem, sweep0, nsweeps, kT, 32, trace_k, stream);
+        if (st != SMC_OK || (!e_acc && !n_acc)) return st;
+        return launch_lc_reduce(P.part_e, P.part_n, nc, scr + off_red, e_acc, (long long *)n_acc, stream);
+    }
     P.dE_out = trace_dE;
     P.acc_out = trace_acc;
     for (int t = 0; t < nsweeps; ++t) {
