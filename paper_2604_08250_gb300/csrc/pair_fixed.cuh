@@ -229,4 +229,17 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
                                       cudaStream_t stream);
 int debug_resident();
 
+// The sweep of small boxes by one CTA per replica (sweep_cta.cu):
+// SMC_ERR_UNSUPPORTED, with nothing enqueued, when a replica does not fit it.
+// most: trials per mini-step up to which it is taken (at most kCtaMaxTrials);
+// check: report species outside [0, S).
+constexpr int kCtaMaxTrials = 128;
+smc_status launch_pair_sweep_cta(int R, const smc_lattice *lats, const smc_model *m, const PairTable &pt,
+                                 int8_t *const *occ, uint64_t seed, uint32_t replica0, uint64_t sweep0, int nsweeps,
+                                 const double *kT, int most, bool check, double *e_acc, int64_t *n_acc,
+                                 cudaStream_t stream);
+
+// Exponent factor of the FP Metropolis test: -log2(e) 2^-sigma / kT.
+inline float accept_cx(double scale, double kT) { return (float)(-1.4426950408889634 * scale / kT); }
+
 }  // namespace smc

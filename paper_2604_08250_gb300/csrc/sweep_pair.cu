@@ -1618,12 +1618,6 @@ bool build_pair_table(const smc_model *m, int S, PairTable &t)
     return true;
 }
 
-// Exponent factor of the FP Metropolis test: -log2(e) 2^-sigma / kT.
-static float accept_cx(double scale, double kT)
-{
-    return (float)(-1.4426950408889634 * scale / kT);
-}
-
 static void load_table(SweepParams &P, const PairTable &pt)
 {
     P.qrow = pt.rw;
@@ -2103,16 +2097,36 @@ static smc_status sweep_impl(int R, const smc_lattice *lats, const smc_model *m,
         set_error("pair coefficients must be finite");
         return SMC_ERR_ARG;
     }
+    int rowB = 0;
+    const bool fast = fast_ok(R, lats, occ, rowB);
+    // Small boxes run in one CTA each (sweep_cta.cu), boxes whose rows fit the
+    // SMs' shared memory resident there (sweep_resident.cu).  Measured per sweep
+    // (two shells, FP32): 8^3 cells 38 us in one CTA against 165 streaming; 12^3
+    // 48 against 60 resident, 16^3 61 and 62, 20^3 93 and 63; sixty-four 20^3
+    // replicas 100 against 304 (the resident kernel takes them in waves); boxes
+    // with an axis that is no multiple of four, one trial per mini-step along
+    // it, 8 to 20 times less than the general kernel.
+    const bool cta = debug_resident() == 0 && debug_skip_tile() < 0;
+    auto one_cta = [&](int most) {
+        return launch_pair_sweep_cta(R, lats, m, pt, occ, seed, replica0, sweep0, nsweeps, kT, most, fast, e_acc, n_acc,
+                                     stream);
+    };
+    if (cta) {
+        st = one_cta(!fast || R >= 16 ? kCtaMaxTrials : 48);
+        if (st != SMC_ERR_UNSUPPORTED) return st;
+    }
     if (debug_resident() == 0) {
         // lattices that fit in the SMs' shared memory stay there
         st = launch_pair_sweep_resident(R, lats, m, pt, occ, seed, replica0, sweep0, nsweeps, kT, e_acc, n_acc,
                                         stream);
         if (st != SMC_ERR_UNSUPPORTED) return st;
     }
-    int rowB = 0;
-    const bool fast = fast_ok(R, lats, occ, rowB);
     // (paired kernel: bulk row copies, so 16-byte aligned rows)
     const bool wide = fast && fast_wide(R, lats, pt.nsh, pt.sw) && (uintptr_t)occ[0] % 16 == 0;
+    if (cta && !wide) {  // boxes that the resident kernel does not take (two link cells along y or z): 92 against 178 us
+        st = one_cta(kCtaMaxTrials);
+        if (st != SMC_ERR_UNSUPPORTED) return st;
+    }
     Plan pl;
     if (wide)
         st = make_pairs_plan<IS_INT>(lats[0], ws, pl);
