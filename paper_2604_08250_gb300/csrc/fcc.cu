@@ -48,6 +48,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "planes.cuh"
 #include "qsro_group.cuh"
 
 namespace smc {
@@ -1076,10 +1077,19 @@ smc_status launch_fcc_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
                                    : (is_int ? pick_fcc<true>(m->nshells) : pick_fcc<false>(m->nshells));
     if (is_qsro) {  // the count cache, from the occupancy at the start of every call
         P.qcache = scr + off_q;
-        const int cb = (int)std::max<size_t>(1, std::min<size_t>((N + 255) / 256, (size_t)ws->num_sms * 16));
-        k_fcc_qsro_cache<<<cb, 256, 0, stream>>>(static_cast<const FccStep &>(P));
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return cuda_fail(e, "k_fcc_qsro_cache");
+        Planes pl;
+        if ((long long)N >= kPlanesMinSites &&
+            planes_build(kPlanesFcc, lat->nx, lat->ny, lat->nz, occ, ws->num_sms, pl, &st, stream)) {
+            st = planes_own(pl, m->nshells, P.qcache, nullptr, stream);
+            if (st != SMC_OK) return st;
+        } else if (st != SMC_OK) {
+            return st;
+        } else {
+            const int cb = (int)std::max<size_t>(1, std::min<size_t>((N + 255) / 256, (size_t)ws->num_sms * 16));
+            k_fcc_qsro_cache<<<cb, 256, 0, stream>>>(static_cast<const FccStep &>(P));
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return cuda_fail(e, "k_fcc_qsro_cache");
+        }
     }
     if (qgrouped) {
         gq.seed = seed;
@@ -1133,10 +1143,21 @@ smc_status launch_fcc_energy(const smc_lattice *lat, const smc_model *m, const i
     const bool is_qsro = m->kind == SMC_QSRO_F32;
     if (is_qsro) P.qcache = cnt;  // marks the qSRO energy (not dereferenced)
     const long long N = 4LL * lat->nx * lat->ny * lat->nz;
-    const int blocks = (int)std::max(1LL, std::min<long long>((N + 255) / 256, (long long)ws->num_sms * 8));
-    k_fcc_pair_counts<<<blocks, 256, 0, stream>>>(P, cnt, is_qsro ? cnt + kMaxShells * 64 : nullptr);
-    err = cudaGetLastError();
-    if (err != cudaSuccess) return cuda_fail(err, "k_fcc_pair_counts");
+    // (planes: a neighbour's cell lies within one box length, so every axis needs two cells)
+    Planes pl;
+    const bool planes = N >= kPlanesMinSites && lat->nx >= 2 && lat->ny >= 2 && lat->nz >= 2 &&
+                        planes_build(kPlanesFcc, lat->nx, lat->ny, lat->nz, occ, ws->num_sms, pl, &st, stream);
+    if (st != SMC_OK) return st;
+    if (planes) {
+        st = planes_pairs(pl, m->nshells, P.S, cnt, stream);
+        if (st == SMC_OK && is_qsro) st = planes_own(pl, m->nshells, nullptr, cnt + kMaxShells * 64, stream);
+        if (st != SMC_OK) return st;
+    } else {
+        const int blocks = (int)std::max(1LL, std::min<long long>((N + 255) / 256, (long long)ws->num_sms * 8));
+        k_fcc_pair_counts<<<blocks, 256, 0, stream>>>(P, cnt, is_qsro ? cnt + kMaxShells * 64 : nullptr);
+        err = cudaGetLastError();
+        if (err != cudaSuccess) return cuda_fail(err, "k_fcc_pair_counts");
+    }
     k_fcc_energy_finish<<<1, 32, 0, stream>>>(P, cnt, m->kind == SMC_PAIR_I32 ? 1 : 0, m->unit_ev, e,
                                               (long long *)e_int);
     err = cudaGetLastError();

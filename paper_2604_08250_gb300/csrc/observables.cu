@@ -12,6 +12,7 @@
 #include <cstdint>
 
 #include "smc_common.cuh"
+#include "planes.cuh"
 
 namespace smc {
 
@@ -383,33 +384,10 @@ __global__ void __launch_bounds__(256) k_pair_counts_planes(const uint4 *__restr
     }
 }
 
-// A grow-only device buffer for the planes (kept apart from the workspace,
-// whose scratch the callers already use for the counts).
-void *planes_buffer(size_t bytes, smc_status *st)
+void launch_planes_aligned(const int8_t *occ, long long nwords, uint4 *planes, int num_sms, cudaStream_t stream)
 {
-    static void *buf = nullptr;
-    static size_t cap = 0;
-    static int dev = -1;
-    int d = 0;
-    cudaError_t e = cudaGetDevice(&d);
-    if (e != cudaSuccess) {
-        *st = cuda_fail(e, "cudaGetDevice");
-        return nullptr;
-    }
-    if (buf && (bytes <= cap) && d == dev) return buf;
-    e = cudaDeviceSynchronize();
-    if (e == cudaSuccess && buf) e = cudaFree(buf);
-    buf = nullptr;
-    cap = 0;
-    if (e == cudaSuccess) e = cudaMalloc(&buf, bytes);
-    if (e != cudaSuccess) {
-        buf = nullptr;
-        *st = cuda_fail(e, "cudaMalloc(planes)");
-        return nullptr;
-    }
-    cap = bytes;
-    dev = d;
-    return buf;
+    const int grid = (int)std::max(1LL, std::min<long long>((nwords + 255) / 256, (long long)num_sms * 8));
+    k_planes<<<grid, 256, 0, stream>>>(occ, nwords, planes);
 }
 
 template <int NSH, int S>
@@ -466,14 +444,21 @@ smc_status launch_pair_counts(const smc_lattice *lat, int nshells, const int8_t 
         S * (S + 1) / 2 * nshells <= 84) {
         const int nw = lat->nx / 32;
         const long long nwords = rows * nw;
-        uint4 *planes = (uint4 *)planes_buffer((size_t)nwords * sizeof(uint4), &st);
-        if (!planes) return st;
-        const int grid = (int)std::max(1LL, std::min<long long>((nwords + 255) / 256, (long long)ws->num_sms * 8));
-        k_planes<<<grid, 256, 0, stream>>>(occ, nwords, planes);
-        if (planes_counts(nshells, S, ws->num_sms * 4, planes, nw, lat->ny, lat->nz, counts, stream)) {
-            e = cudaGetLastError();
-            return e == cudaSuccess ? SMC_OK : cuda_fail(e, "k_pair_counts_planes");
+        uint4 *planes = (uint4 *)planes_buffer((size_t)nwords * sizeof(uint4), stream);
+        if (planes) {
+            launch_planes_aligned(occ, nwords, planes, ws->num_sms, stream);
+            if (planes_counts(nshells, S, ws->num_sms * 4, planes, nw, lat->ny, lat->nz, counts, stream)) {
+                e = cudaGetLastError();
+                return e == cudaSuccess ? SMC_OK : cuda_fail(e, "k_pair_counts_planes");
+            }
         }
+    }
+    // other rows (and three shells of eight species): 200 x 120 x 88 cells, 3 shells, 8 species, 0.27 ms by bytes
+    if (rows * lat->nx >= kPlanesMinSites) {
+        Planes P;
+        if (planes_build(kPlanesBcc, lat->nx, lat->ny, lat->nz, occ, ws->num_sms, P, &st, stream))
+            return planes_pairs(P, nshells, S, counts, stream);
+        if (st != SMC_OK) return st;
     }
     const int threads = 256;
     const long long want = (rows + 7) / 8;

@@ -31,6 +31,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "planes.cuh"
 #include "qsro_group.cuh"
 
 namespace smc {
@@ -591,9 +592,18 @@ smc_status launch_qsro_ministeps(const smc_lattice *lat, const smc_model *m, int
     const int blocks = P.bnd_blocks + (P.n_int + threads - 1) / threads;
     const BqKernel kern = m->nshells == 1 ? k_bq_ministep<1> : (m->nshells == 2 ? k_bq_ministep<2> : k_bq_ministep<3>);
     const int cb = (int)std::max<size_t>(1, std::min<size_t>((N + 255) / 256, (size_t)ws->num_sms * 16));
-    k_bq_cache<<<cb, 256, 0, stream>>>(P);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "k_bq_cache");
+    Planes pl;
+    if ((long long)N >= kPlanesMinSites &&
+        planes_build(kPlanesBcc, lat->nx, lat->ny, lat->nz, occ, ws->num_sms, pl, &st, stream)) {
+        st = planes_own(pl, m->nshells, P.qcache, nullptr, stream);
+        if (st != SMC_OK) return st;
+    } else if (st != SMC_OK) {
+        return st;
+    } else {
+        k_bq_cache<<<cb, 256, 0, stream>>>(P);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(e, "k_bq_cache");
+    }
     if (grouped) {
         gp.seed = seed;
         gp.replica = replica;

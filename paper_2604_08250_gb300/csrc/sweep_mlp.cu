@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "mlp_zone.cuh"
+#include "planes.cuh"
 
 namespace smc {
 
@@ -1134,7 +1135,12 @@ smc_status qsro_counts_finish(const smc_lattice *lat, const smc_model *m, const 
     if (st != SMC_OK) return st;
     cudaError_t err = cudaMemsetAsync(quad, 0, sizeof(unsigned long long) * kMaxShells * kMaxSpecies, stream);
     if (err != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync(qSRO sums)");
-    st = qsro_sites_launch(ws, lat, m->nshells, occ, quad, stream);
+    Planes pl;
+    if (2LL * lat->nx * lat->ny * lat->nz >= kPlanesMinSites &&
+        planes_build(kPlanesBcc, lat->nx, lat->ny, lat->nz, occ, ws->num_sms, pl, &st, stream))
+        st = planes_own(pl, m->nshells, nullptr, quad, stream);
+    else if (st == SMC_OK)
+        st = qsro_sites_launch(ws, lat, m->nshells, occ, quad, stream);
     if (st != SMC_OK) return st;
     const long long N = 2LL * lat->nx * lat->ny * lat->nz;
     k_qsro_finish<<<1, 32, 0, stream>>>(make_qsro_raw(m, lat->nspecies), cnt, quad, N, e, grad);
