@@ -596,27 +596,30 @@ __global__ void __launch_bounds__(256) k_fcc_pair_counts(const __grid_constant__
 __global__ void k_fcc_energy_finish(const __grid_constant__ FccParams P, const unsigned long long *counts, int is_int,
                                     double unit, double *e, long long *e_int)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int n = P.nshells * P.S * P.S;
+    // one warp: lane l takes the terms l, l + 32, ...
+    const int n = P.nshells * P.S * P.S, lane = threadIdx.x;
     if (is_int) {
         long long tot = 0;
-        for (int i = 0; i < n; ++i) tot += (long long)P.vi[i] * (long long)counts[i];
-        tot /= 2;  // every bond counted from both ends
-        if (e_int) *e_int = tot;
-        if (e) *e = (double)tot * unit;
+        for (int i = lane; i < n; i += 32) tot += (long long)P.vi[i] * (long long)counts[i];
+        tot = warp_sum<long long>(tot) / 2;  // every bond counted from both ends
+        if (lane == 0 && e_int) *e_int = tot;
+        if (lane == 0 && e) *e = (double)tot * unit;
     } else if (e && P.qcache) {  // qSRO: E = N C + sum V n / z_m + sum W Q / z_m^2
         const double z[3] = {12.0, 6.0, 24.0};
         const unsigned long long *sq = counts + kMaxShells * 64;
-        double tot = 4.0 * P.nx * P.ny * P.nz * P.qc;
-        for (int i = 0; i < n; ++i) tot += (double)P.vf[i] * (double)counts[i] / z[i / (P.S * P.S)];
-        for (int m = 0; m < P.nshells; ++m)
-            for (int p = 0; p < P.S; ++p)
-                tot += (double)P.wq[m * P.S + p] * (double)sq[m * kMaxSpecies + p] / (z[m] * z[m]);
-        *e = tot;
+        double tot = 0.0;
+        for (int i = lane; i < n; i += 32) tot += (double)P.vf[i] * (double)counts[i] / z[i / (P.S * P.S)];
+        for (int i = lane; i < P.nshells * P.S; i += 32) {
+            const int m = i / P.S;
+            tot += (double)P.wq[i] * (double)sq[m * kMaxSpecies + i % P.S] / (z[m] * z[m]);
+        }
+        tot = warp_sum<double>(tot);
+        if (lane == 0) *e = 4.0 * P.nx * P.ny * P.nz * P.qc + tot;
     } else if (e) {
         double tot = 0.0;
-        for (int i = 0; i < n; ++i) tot += (double)P.vf[i] * (double)counts[i];
-        *e = 0.5 * tot;
+        for (int i = lane; i < n; i += 32) tot += (double)P.vf[i] * (double)counts[i];
+        tot = warp_sum<double>(tot);
+        if (lane == 0) *e = 0.5 * tot;
     }
 }
 

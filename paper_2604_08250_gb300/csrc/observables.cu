@@ -521,22 +521,24 @@ struct VBlock {
     float vf[kMaxShells * kMaxSpecies * kMaxSpecies];
 };
 
+// One warp: lane l adds the terms l, l + 32, ..., then a fixed tree (a single
+// thread took 10 us for 50 terms, 30 for 192).
 __global__ void k_energy_finish(VBlock V, int is_int, int nshells, int S, const unsigned long long *counts,
                                 double *e, long long *e_int, double *e_add)
 {
-    if (threadIdx.x != 0) return;
+    const int lane = threadIdx.x, n = nshells * S * S;
     if (is_int) {
         long long tot = 0;
-        for (int i = 0; i < nshells * S * S; ++i) tot += (long long)V.vi[i] * (long long)counts[i];
-        tot /= 2;  // every bond is counted from both ends
-        if (e_int) *e_int = tot;
-        if (e) *e = (double)tot;
+        for (int i = lane; i < n; i += 32) tot += (long long)V.vi[i] * (long long)counts[i];
+        tot = warp_sum<long long>(tot) / 2;  // every bond is counted from both ends
+        if (lane == 0 && e_int) *e_int = tot;
+        if (lane == 0 && e) *e = (double)tot;
     } else {
         double tot = 0.0;
-        for (int i = 0; i < nshells * S * S; ++i) tot = __dadd_rn(tot, __dmul_rn((double)V.vf[i], (double)counts[i]));
-        tot = __dmul_rn(0.5, tot);
-        if (e_add) tot = __dadd_rn(tot, *e_add);
-        if (e) *e = tot;
+        for (int i = lane; i < n; i += 32) tot = __dadd_rn(tot, __dmul_rn((double)V.vf[i], (double)counts[i]));
+        tot = __dmul_rn(0.5, warp_sum<double>(tot));
+        if (lane == 0 && e_add) tot = __dadd_rn(tot, *e_add);
+        if (lane == 0 && e) *e = tot;
     }
 }
 

@@ -123,14 +123,6 @@ __device__ __forceinline__ bool metropolis(typename Acc<IS_INT>::T dE, uint32_t 
     }
 }
 
-template <typename V>
-__device__ __forceinline__ V warp_sum(V v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 extern __shared__ __align__(16) unsigned char g_smem[];
 
 #define SM8(off) ((uint32_t)g_smem[(off)])

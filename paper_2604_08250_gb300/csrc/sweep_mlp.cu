@@ -107,12 +107,13 @@ __global__ void __launch_bounds__(128 * kStreamWG) k_mlp_site_energy(const void 
     tc_teardown(E, NWG);
 }
 
-// out (+)= sum of part[0 .. n-1], in index order.
+// out (+)= sum of part[0 .. n-1] in a fixed order, by one warp.
 __global__ void k_sum_parts(const double *part, int n, double *out, int accumulate)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
     double s = 0.0;
-    for (int i = 0; i < n; ++i) s += part[i];
+    for (int i = threadIdx.x; i < n; i += 32) s += part[i];
+    s = warp_sum<double>(s);
+    if (threadIdx.x != 0) return;
     if (accumulate)
         *out += s;
     else
@@ -594,30 +595,39 @@ struct QsroRaw {
 __global__ void k_qsro_finish(QsroRaw Q, const unsigned long long *cnt, const unsigned long long *quad, long long N,
                               double *e, float *grad)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    // one warp: lane l takes terms and parameters l, l + 32, ...
     const double z[3] = {8.0, 6.0, 12.0};
-    const int S = Q.S;
+    const int S = Q.S, nv = Q.nsh * S * S, lane = threadIdx.x;
     if (e) {
         double E = 0.0;
-        for (int m = 0; m < Q.nsh; ++m)
-            for (int p = 0; p < S; ++p)
-                for (int q = 0; q < S; ++q) E += Q.v[m][p][q] * (double)cnt[(m * S + p) * S + q] / z[m];
-        for (int m = 0; m < Q.nsh; ++m)
-            for (int p = 0; p < S; ++p) E += Q.w[m][p] * (double)quad[m * kMaxSpecies + p] / (z[m] * z[m]);
-        *e = E + (double)N * Q.c;
+        for (int i = lane; i < nv; i += 32) {
+            const int m = i / (S * S), p = (i / S) % S, q = i % S;
+            E += Q.v[m][p][q] * (double)cnt[i] / z[m];
+        }
+        for (int i = lane; i < Q.nsh * S; i += 32) {
+            const int m = i / S, p = i % S;
+            E += Q.w[m][p] * (double)quad[m * kMaxSpecies + p] / (z[m] * z[m]);
+        }
+        E = warp_sum<double>(E);
+        if (lane == 0) *e = E + (double)N * Q.c;
     }
     if (grad) {
-        int i = 0;
-        for (int m = 0; m < Q.nsh; ++m)
-            for (int p = 0; p < S; ++p)
-                for (int q = p; q < S; ++q) {
-                    const double n = p == q ? (double)cnt[(m * S + p) * S + p]
-                                            : (double)cnt[(m * S + p) * S + q] + (double)cnt[(m * S + q) * S + p];
-                    grad[i++] = (float)(n / z[m]);
-                }
-        for (int m = 0; m < Q.nsh; ++m)
-            for (int p = 0; p < S; ++p) grad[i++] = (float)((double)quad[m * kMaxSpecies + p] / (z[m] * z[m]));
-        grad[i] = (float)N;
+        const int per = S * (S + 1) / 2;
+        for (int i = lane; i < Q.nsh * per; i += 32) {
+            const int m = i / per;
+            int r = i % per, p = 0;
+            while (r >= S - p) {
+                r -= S - p;
+                ++p;
+            }
+            const int q = p + r;
+            const double n = p == q ? (double)cnt[(m * S + p) * S + p]
+                                    : (double)cnt[(m * S + p) * S + q] + (double)cnt[(m * S + q) * S + p];
+            grad[i] = (float)(n / z[m]);
+        }
+        for (int i = lane; i < Q.nsh * S; i += 32)
+            grad[Q.nsh * per + i] = (float)((double)quad[(i / S) * kMaxSpecies + i % S] / (z[i / S] * z[i / S]));
+        if (lane == 0) grad[Q.nsh * (per + S)] = (float)N;
     }
 }
 
