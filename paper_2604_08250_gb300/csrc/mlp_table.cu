@@ -184,6 +184,37 @@ struct TableParams {
     long long timeout_ns;
 };
 
+// Table index of a site word.  Plain rank order spreads the probable vectors
+// over the whole of the five-species table, 3.8 GB: a random alloy finds half
+// of its look-ups in 256 of the 1900 2 MB pages.  There (SPLIT) every shell's
+// ranks are cut into probable and other ones, and the eight combinations lie
+// one after the other, the most probable first: 50 % of the look-ups in 98
+// pages, and a group of mini-steps at 256^3 takes 0.70 ms instead of 0.80
+// (cuts at 64, 48, 400 and 96, 96, 768: 0.71 and 0.72).  A finer cut by digits
+// with a table of places took 0.76, one by bit fields 0.80 (its power-of-two
+// strides crowd the cache sets).
+constexpr uint32_t kCut1 = 96, kCut2 = 64, kCut3 = 512;
+constexpr uint32_t kRest1 = 495 - kCut1, kRest2 = 210 - kCut2, kRest3 = 1820 - kCut3;
+
+template <bool SPLIT>
+__device__ __forceinline__ uint32_t word_index(const TableDims &D, uint32_t w)
+{
+    const uint32_t s = w >> kWordSp, r1 = (w >> word_sh(0)) & word_mask(0), r2 = (w >> word_sh(1)) & word_mask(1),
+                   r3 = w & word_mask(2);
+    if (!SPLIT) return ((s * (uint32_t)D.n[0] + r1) * (uint32_t)D.n[1] + r2) * (uint32_t)D.n[2] + r3;
+    constexpr uint32_t a1 = kCut1, a2 = kCut2, a3 = kCut3, b1 = kRest1, b2 = kRest2, b3 = kRest3;
+    // starts of the combinations (shell 1, 2, 3 beyond its cut)
+    constexpr uint32_t z001 = 5 * a1 * a2 * a3, z010 = z001 + 5 * a1 * a2 * b3, z100 = z010 + 5 * a1 * b2 * a3,
+                       z011 = z100 + 5 * b1 * a2 * a3, z101 = z011 + 5 * a1 * b2 * b3, z110 = z101 + 5 * b1 * a2 * b3,
+                       z111 = z110 + 5 * b1 * b2 * a3;
+    static_assert((unsigned long long)z111 + 5ull * b1 * b2 * b3 == 5ull * 495 * 210 * 1820, "the blocks fill the table");
+    const bool c1 = r1 >= a1, c2 = r2 >= a2, c3 = r3 >= a3;
+    const uint32_t d1 = c1 ? b1 : a1, d2 = c2 ? b2 : a2, d3 = c3 ? b3 : a3;
+    const uint32_t q1 = c1 ? r1 - a1 : r1, q2 = c2 ? r2 - a2 : r2, q3 = c3 ? r3 - a3 : r3;
+    const uint32_t z = c1 ? (c2 ? (c3 ? z111 : z110) : (c3 ? z101 : z100)) : (c2 ? (c3 ? z011 : z010) : (c3 ? z001 : 0u));
+    return z + ((s * d1 + q1) * d2 + q2) * d3 + q3;
+}
+
 // ---------------------------------------------------------------------------
 // f of every feature vector.  Tile t holds vectors 128 t .. 128 t + 127.
 // ---------------------------------------------------------------------------
@@ -197,10 +228,11 @@ __global__ void __launch_bounds__(128 * kStreamWG) k_table_fill(const void *W, c
     mlp_cta_setup<Net, NWG>(E, W, nullptr, nullptr);
     const int r = threadIdx.x & 127, wg = threadIdx.x >> 7;
     const uint32_t nv = (uint32_t)D.entries, ntile = (nv + kTcRows - 1) / kTcRows;
+    // features of vector 128 tl + r; its place in the table (~0: past the last)
     auto build = [&](uint32_t tl) {
         const uint32_t v = tl * kTcRows + r;
         int q0 = -1;
-        uint32_t h1 = 0, h2 = 0, h3 = 0;
+        uint32_t h1 = 0, h2 = 0, h3 = 0, at = ~0u;
         if (v < nv) {
             const uint32_t t3 = v / (uint32_t)D.n[2], r3 = v - t3 * (uint32_t)D.n[2];
             const uint32_t t2 = t3 / (uint32_t)D.n[1], r2 = t3 - t2 * (uint32_t)D.n[1];
@@ -209,36 +241,33 @@ __global__ void __launch_bounds__(128 * kStreamWG) k_table_fill(const void *W, c
             h1 = __ldg(unrank + D.un[0] + r1);
             h2 = __ldg(unrank + D.un[1] + r2);
             h3 = __ldg(unrank + D.un[2] + r3);
+            at = D.S == 5 ? word_index<true>(D, t1 << kWordSp | r1 << word_sh(0) | r2 << word_sh(1) | r3) : v;
         }
         tc_write_features(E.L, r, q0, h1, h2, h3);
         fence_async_smem();
+        return at;
     };
     const uint32_t step = (uint32_t)NWG * gridDim.x;
     uint32_t tl = (uint32_t)NWG * blockIdx.x + wg;
+    uint32_t at = ~0u;
     if (tl < ntile) {
-        build(tl);
+        at = build(tl);
         tc_issue1(E);
     }
     while (tl < ntile) {
         tc_stage2(E);
         const uint32_t next = tl + step;
+        uint32_t at_next = ~0u;
         if (next < ntile) {
-            build(next);
+            at_next = build(next);
             tc_issue1(E);
         }
         const float f = tc_finish(E);
-        const uint32_t v = tl * kTcRows + r;
-        if (v < nv) table[v] = f;
+        if (at != ~0u) table[at] = f;
+        at = at_next;
         tl = next;
     }
     tc_teardown(E, NWG);
-}
-
-__device__ __forceinline__ uint32_t word_index(const TableDims &D, uint32_t w)
-{
-    const uint32_t s = w >> kWordSp, r1 = (w >> word_sh(0)) & word_mask(0), r2 = (w >> word_sh(1)) & word_mask(1),
-                   r3 = w & word_mask(2);
-    return ((s * (uint32_t)D.n[0] + r1) * (uint32_t)D.n[1] + r2) * (uint32_t)D.n[2] + r3;
 }
 
 // Position of cell x in a row of states: cells of one residue x mod 4 are
@@ -273,7 +302,7 @@ __global__ void __launch_bounds__(256) k_table_state(const __grid_constant__ Tab
             }
             w |= (uint32_t)__ldg(P.ranks + P.d.rk[m] + v) << word_sh(m);
         }
-        P.state[s - x + state_pos(x, P.NLx)] = make_uint2(w, __float_as_uint(__ldg(P.table + word_index(P.d, w))));
+        P.state[s - x + state_pos(x, P.NLx)] = make_uint2(w, __float_as_uint(__ldg(P.table + (S == 5 ? word_index<true>(P.d, w) : word_index<false>(P.d, w)))));
     }
 }
 
@@ -343,7 +372,7 @@ __device__ __forceinline__ void team_sync(int team, int n)
     asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(n) : "memory");
 }
 
-template <bool HAS_PAIR>
+template <bool HAS_PAIR, bool SPLIT>
 __global__ void __launch_bounds__(kTabThreads, 1) k_table_sweep(const __grid_constant__ TableParams P)
 {
     // shared memory: moves | zone table | the moves' offsets | progress | (pair) D | per team: row numbers,
@@ -447,7 +476,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_table_sweep(const __grid_con
                         if (k == 0 && sl < 2)  // a, b themselves
                             w = (w & ((1u << kWordSp) - 1u)) | (sl == 0 ? B : A) << kWordSp;
                         nw[k] = w;
-                        nf[k] = __ldg(P.table + word_index(P.d, w));
+                        nf[k] = __ldg(P.table + word_index<SPLIT>(P.d, w));
                     }
                 }
 #pragma unroll
@@ -642,7 +671,8 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
     k_table_state<<<sb, 256, 0, stream>>>(P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "k_table_state");
-    auto kern = pair ? k_table_sweep<true> : k_table_sweep<false>;
+    auto kern = T.d.S == 5 ? (pair ? k_table_sweep<true, true> : k_table_sweep<false, true>)
+                           : (pair ? k_table_sweep<true, false> : k_table_sweep<false, false>);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_table_sweep)");
     const int blocks = std::min(P.ncol, ws->num_sms), threads = P.team_threads * P.K;
