@@ -298,12 +298,10 @@ static __device__ void tc_teardown(TcEval &E, int nwg)
     if (threadIdx.x < 32) tc_dealloc(*(const uint32_t *)(g_smem + E.L.tmem_slot), kTcCols * nwg);
 }
 
-// Writes the features of row r into the X tile (q0 < 0 and zero histograms
-// give a row of zeros).
-__device__ __forceinline__ void tc_write_features(const TcLayout &L, uint32_t r, int q0, uint32_t h1, uint32_t h2,
-                                                  uint32_t h3)
+// The feature row of a site, 32 BF16 values (q0 < 0 and zero histograms give
+// zeros and the three ones).
+__device__ __forceinline__ void tc_feature_words(int q0, uint32_t h1, uint32_t h2, uint32_t h3, uint32_t (&w)[16])
 {
-    uint32_t w[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
         float v[2];
@@ -325,6 +323,14 @@ __device__ __forceinline__ void tc_write_features(const TcLayout &L, uint32_t r,
         }
         w[c] = pack_bf16(v[0], v[1]);
     }
+}
+
+// Writes the features of row r into the X tile.
+__device__ __forceinline__ void tc_write_features(const TcLayout &L, uint32_t r, int q0, uint32_t h1, uint32_t h2,
+                                                  uint32_t h3)
+{
+    uint32_t w[16];
+    tc_feature_words(q0, h1, h2, h3, w);
 #pragma unroll
     for (int kc = 0; kc < 4; ++kc)
         *(uint4 *)(g_smem + L.x + tc_off32(r, kc)) = make_uint4(w[4 * kc], w[4 * kc + 1], w[4 * kc + 2], w[4 * kc + 3]);
