@@ -8,6 +8,7 @@ loading fails loudly otherwise -- there is no CPU fallback.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 
 import numpy as np
@@ -112,7 +113,15 @@ def _chk(code: int):
 
 def _stream():
     import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+
+
+_PTR = {t: C.POINTER(t) for t in (C.c_int32, C.c_float, C.c_uint16)}
+
+
+def _ptr(a, ctype):
+    """Typed pointer to a contiguous array that the caller keeps (a third of the cost of ndarray.ctypes.data_as)."""
+    return C.cast(a.__array_interface__["data"][0], _PTR[ctype])
 
 
 def _dptr(t, dtype=None):
@@ -153,31 +162,31 @@ class Model:
         c.kind, c.nshells, c.unit_ev = self.kind, self.nshells, self.unit_ev
         if kind == PAIR_I32:
             self.v = np.ascontiguousarray(v, dtype=np.int32)
-            c.v_i32 = self.v.ctypes.data_as(C.POINTER(C.c_int32))
+            c.v_i32 = _ptr(self.v, C.c_int32)
         elif kind in (PAIR_F32, PAIR_F32_MLP_BF16, QSRO_F32):
             self.v = np.ascontiguousarray(v, dtype=np.float32)
-            c.v_f32 = self.v.ctypes.data_as(C.POINTER(C.c_float))
+            c.v_f32 = _ptr(self.v, C.c_float)
         if kind == QSRO_F32:
             self.qsro_w = np.ascontiguousarray(qsro_w, dtype=np.float32)
-            c.qsro_w = self.qsro_w.ctypes.data_as(C.POINTER(C.c_float))
+            c.qsro_w = _ptr(self.qsro_w, C.c_float)
             c.qsro_c = float(qsro_c)
         if kind == MLPNET_BF16:  # net: w0..w3 BF16 bit patterns, b0..b2 FP32, b3
             self.net = {k: np.ascontiguousarray(net[k], dtype=np.uint16).reshape(-1) for k in ("w0", "w1", "w2", "w3")}
             for k in ("b0", "b1", "b2"):
                 self.net[k] = np.ascontiguousarray(net[k], dtype=np.float32).reshape(-1)
             for k in ("w0", "w1", "w2", "w3"):
-                setattr(c, "net_" + k, self.net[k].ctypes.data_as(C.POINTER(C.c_uint16)))
+                setattr(c, "net_" + k, _ptr(self.net[k], C.c_uint16))
             for k in ("b0", "b1", "b2"):
-                setattr(c, "net_" + k, self.net[k].ctypes.data_as(C.POINTER(C.c_float)))
+                setattr(c, "net_" + k, _ptr(self.net[k], C.c_float))
             c.net_b3 = float(net["b3"])
         if kind in (MLP_BF16, PAIR_F32_MLP_BF16):
             self.mlp = {k: np.ascontiguousarray(mlp[k], dtype=np.uint16).reshape(-1) for k in ("w1", "w2", "w3")}
             for k in ("b1", "b2"):
                 self.mlp[k] = np.ascontiguousarray(mlp[k], dtype=np.float32).reshape(-1)
             for k in ("w1", "w2", "w3"):
-                setattr(c, "mlp_" + k, self.mlp[k].ctypes.data_as(C.POINTER(C.c_uint16)))
+                setattr(c, "mlp_" + k, _ptr(self.mlp[k], C.c_uint16))
             for k in ("b1", "b2"):
-                setattr(c, "mlp_" + k, self.mlp[k].ctypes.data_as(C.POINTER(C.c_float)))
+                setattr(c, "mlp_" + k, _ptr(self.mlp[k], C.c_float))
             c.mlp_b3 = float(mlp["b3"])
         self._c = c
 
@@ -306,9 +315,17 @@ def debug_set(what, value):
 # ---------------------------------------------------------------------------
 def _bf16_bits(a):
     """float -> BF16 bit patterns, round to nearest even (through FP32)."""
-    u = np.ascontiguousarray(a, dtype=np.float32).view(np.uint32).astype(np.uint64)
-    u = (u + 0x7FFF + ((u >> 16) & 1)) >> 16
-    return u.astype(np.uint16)
+    u = np.ascontiguousarray(a, dtype=np.float32).view(np.uint32)
+    r = (u >> 16) & 1
+    r += 0x7FFF
+    r += u  # modulo 2^32: only bits 16-31 are kept
+    r >>= 16
+    return r.astype(np.uint16)
+
+
+@functools.lru_cache(maxsize=8)
+def _upper(S):
+    return np.triu_indices(S)
 
 
 def n_pair_params(nshells, S):
@@ -325,22 +342,21 @@ def model_from_theta(kind, nshells, S, theta):
     v = None
     if kind in (PAIR_F32, PAIR_F32_MLP_BF16):
         v = np.zeros((nshells, S, S), dtype=np.float32)
-        for m in range(nshells):
-            for p in range(S):
-                for q in range(p, S):
-                    v[m, p, q] = v[m, q, p] = th[k]
-                    k += 1
+        k = n_pair_params(nshells, S)
+        if k > th.size:
+            raise IndexError(f"theta has {th.size} entries, the pair part alone needs {k}")
+        p, q = _upper(S)
+        v[:, p, q] = v[:, q, p] = th[:k].reshape(nshells, p.size)
     elif kind != MLP_BF16:
         raise ValueError("parameter vectors are defined for PAIR_F32, MLP_BF16 and PAIR_F32_MLP_BF16 models")
     mlp = None
     if kind in (MLP_BF16, PAIR_F32_MLP_BF16):
         sizes = (("w1", 64 * 20), ("b1", 64), ("w2", 64 * 64), ("b2", 64), ("w3", 64), ("b3", 1))
         mlp = {}
+        bits, k0 = _bf16_bits(th[k:]), k  # of the biases too: one pass costs less than three
         for name, n in sizes:
-            mlp[name] = th[k:k + n]
+            mlp[name] = bits[k - k0:k - k0 + n] if name[0] == "w" else th[k:k + n]
             k += n
-        for name in ("w1", "w2", "w3"):
-            mlp[name] = _bf16_bits(mlp[name])
         mlp["b3"] = float(mlp["b3"][0])
     if k != th.size:
         raise ValueError(f"theta has {th.size} entries, the model needs {k}")
@@ -359,14 +375,14 @@ def _autograd_function():
         def forward(ctx, theta, lat, occ, kind, nshells):
             th = theta.detach().cpu().numpy()
             model = model_from_theta(kind, nshells, lat.nspecies, th)
-            e = torch.zeros(1, dtype=torch.float64, device=occ.device)
+            e = torch.empty(1, dtype=torch.float64, device=occ.device)  # the kernels write all of it, and of g
             energy(lat, model, occ, e)
             ctx.lat, ctx.occ, ctx.model = lat, occ, model
             return e.reshape(()).to(theta.dtype).to(theta.device)
 
         @staticmethod
         def backward(ctx, gout):
-            g = torch.zeros(grad_size(ctx.lat, ctx.model), dtype=torch.float32, device=ctx.occ.device)
+            g = torch.empty(grad_size(ctx.lat, ctx.model), dtype=torch.float32, device=ctx.occ.device)
             energy_grad(ctx.lat, ctx.model, ctx.occ, g)
             return gout * g.to(gout.dtype).to(gout.device), None, None, None, None
 
