@@ -593,7 +593,7 @@ bool mlp_table_wanted(const smc_lattice *lat, int nsweeps)
 
 smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, int8_t *occ, uint64_t seed,
                                   uint32_t replica, uint64_t sweep0, int nsweeps, const double *kT, double *e_acc,
-                                  int64_t *n_acc, const float *D, bool *taken, cudaStream_t stream)
+                                  int64_t *n_acc, const float *D, size_t least, bool *taken, cudaStream_t stream)
 {
     *taken = false;
     smc_status st;
@@ -631,7 +631,7 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
                  o_rk = up(o_mv + T.moves.size() * 2), o_un = up(o_rk + T.ranks.size() * 2),
                  o_zone = up(o_un + T.unrank.size() * 4), o_D = up(o_zone + zone.size() * 4),
                  o_red = up(o_D + kDEntries * 4), o_state = up(o_red + lc_reduce_bytes()), o_tab = up(o_state + N * 8),
-                 need = o_tab + (size_t)T.d.entries * 4;
+                 need = std::max(o_tab + (size_t)T.d.entries * 4, least);
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, need, &st);
     if (!scr) {  // no room for the table: the evaluating sweep needs none
         cudaGetLastError();

@@ -185,9 +185,11 @@ smc_status mlp_copy_weights(const smc_model *m, void *dst, cudaStream_t stream);
 // call is large enough for it, and the call; *taken is false when the table
 // does not fit (the caller runs the evaluating sweep).  D: pair table (host).
 bool mlp_table_wanted(const smc_lattice *lat, int nsweeps);
+// (The workspace grows to `least` bytes at least: those of the evaluating
+// sweep, which takes the captured calls that a plain one prepares.)
 smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, int8_t *occ, uint64_t seed,
                                   uint32_t replica, uint64_t sweep0, int nsweeps, const double *kT, double *e_acc,
-                                  int64_t *n_acc, const float *D, bool *taken, cudaStream_t stream);
+                                  int64_t *n_acc, const float *D, size_t least, bool *taken, cudaStream_t stream);
 constexpr size_t kWeightBytes = sizeof(MlpBlock) > sizeof(NetBlock) ? sizeof(MlpBlock) : sizeof(NetBlock);
 
 }  // namespace smc

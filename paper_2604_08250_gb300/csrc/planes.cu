@@ -349,18 +349,19 @@ void own_launch(const Planes &P, int blocks, void *cache, unsigned long long *qu
 
 // The planes' buffer: grown when needed, kept apart from the workspace (whose
 // scratch the callers already use for the counts).  NULL, with nothing
-// changed, while the stream is being captured or without memory.
-void *planes_buffer(size_t bytes, cudaStream_t stream)
+// changed, without memory or when a captured stream would have to grow it.
+// Graphs may hold the buffer of the pair counts of aligned rows (0), so other
+// calls, never captured, grow one of their own (1).
+void *planes_buffer(int which, size_t bytes, cudaStream_t stream)
 {
-    static void *buf = nullptr;
-    static size_t cap = 0;
-    static int dev = -1;
+    static void *bufs[2];
+    static size_t caps[2];
+    static int devs[2] = {-1, -1};
+    void *&buf = bufs[which];
     int d = 0;
     if (cudaGetDevice(&d) != cudaSuccess) return nullptr;
-    if (buf && bytes <= cap && d == dev) return buf;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return nullptr;
-    if (cudaDeviceSynchronize() != cudaSuccess) return nullptr;
+    if (buf && bytes <= caps[which] && d == devs[which]) return buf;
+    if (stream_capturing(stream) || cudaDeviceSynchronize() != cudaSuccess) return nullptr;
     void *p = nullptr;
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -368,8 +369,8 @@ void *planes_buffer(size_t bytes, cudaStream_t stream)
     }
     if (buf) cudaFree(buf);
     buf = p;
-    cap = bytes;
-    dev = d;
+    caps[which] = bytes;
+    devs[which] = d;
     return buf;
 }
 
@@ -377,11 +378,10 @@ bool planes_build(PlaneLattice lat, int nx, int ny, int nz, const int8_t *occ, i
                   cudaStream_t stream)
 {
     *st = SMC_OK;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (stream_capturing(stream)) return false;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    if (dev >= 64 || !g_vec_ready[dev]) {  // the table copy cannot be captured
-        if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
+    if (dev >= 64 || !g_vec_ready[dev]) {
         *st = vec_tables();
         if (*st != SMC_OK) return false;
     }
@@ -392,7 +392,7 @@ bool planes_build(PlaneLattice lat, int nx, int ny, int nz, const int8_t *occ, i
     P.num_sms = num_sms;
     const long long rows = (long long)(lat == kPlanesBcc ? 2 : 4) * ny * nz;
     const int nw = (nx + 31) / 32;
-    uint4 *words = (uint4 *)planes_buffer((size_t)(rows * nw) * sizeof(uint4), stream);
+    uint4 *words = (uint4 *)planes_buffer(1, (size_t)(rows * nw) * sizeof(uint4), stream);
     if (!words) return false;
     P.words = words;
     if (nx % 32 == 0 && (uintptr_t)occ % 16 == 0) {

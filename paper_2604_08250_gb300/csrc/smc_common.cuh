@@ -154,6 +154,14 @@ struct Workspace {
 Workspace *workspace(smc_status *st);
 // Ensures at least `bytes` of scratch after the status header; returns it.
 void *workspace_scratch(Workspace *ws, size_t bytes, smc_status *st);
+// Whether the stream is being captured into a graph (or cannot tell).
+inline bool stream_capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
 
 struct Tuning {
     int tile_y = 0, tile_z = 0, threads = 0, ctas_per_sm = 0;

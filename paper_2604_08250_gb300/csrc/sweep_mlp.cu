@@ -966,15 +966,6 @@ smc_status launch_mlp_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     d.rep = replica;
     d.vec = (d.nx % 16 == 0) && ((uintptr_t)occ % 16 == 0);
     if (has_pair) fill_pair_D(m, P.S, P);
-    // A call whose trials evaluate more rows than there are feature vectors
-    // evaluates each vector once and looks the others up.
-    if (mlp_table_wanted(lat, nsweeps)) {
-        bool taken = false;
-        st = launch_mlp_table_sweep(lat, m, occ, seed, replica, sweep0, nsweeps, kT, e_acc, n_acc, P.D.df, &taken,
-                                    stream);
-        if (st != SMC_OK || taken) return st;
-    }
-
     // workspace: [flags | part_e | part_n | ticket, abort | weights | energy parts | E cache | F cache]
     const size_t nt = (size_t)P.ntiles;
     const size_t N = 2ull * lat->nx * lat->ny * lat->nz;
@@ -984,6 +975,16 @@ smc_status launch_mlp_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     const size_t off_cache =
         round16(off_parts + sizeof(double) * kTcMaxCtasPerSm * (size_t)std::max(ws->num_sms, 1));
     const size_t off_fcache = round16(off_cache + N * 4);
+    // A call whose trials evaluate more rows than there are feature vectors
+    // evaluates each vector once and looks the others up.  Not into a graph:
+    // it would read the host's copies of the tables when it is replayed.
+    if (mlp_table_wanted(lat, nsweeps) && !stream_capturing(stream)) {
+        bool taken = false;
+        st = launch_mlp_table_sweep(lat, m, occ, seed, replica, sweep0, nsweeps, kT, e_acc, n_acc, P.D.df,
+                                    off_fcache + N * 16, &taken, stream);
+        if (st != SMC_OK || taken) return st;
+    }
+
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, off_fcache + N * 16, &st);
     if (!scr) return st;
     P.flags = (uint32_t *)scr;
