@@ -11,8 +11,8 @@
 // a fixed function of the features with the same bits wherever it is
 // evaluated (mlp_tc.cuh), so the looked-up sweep takes the same decisions as
 // the evaluating one.  Measured (GB300, 256^3, five species): the table 35 ms
-// (MLP) or 42 ms (MLPNet), then 25.6 ms per sweep, against 60 ms (MLP) and
-// 90 ms (MLPNet) per sweep of the evaluating kernel.
+// (MLP) or 36 ms (MLPNet), then 22 ms per sweep, against 60 ms (MLP) and 90 ms
+// (MLPNet) per sweep of the evaluating kernel.
 //
 // Feature vectors are numbered shell by shell: r_m is the rank of the shell's
 // composition among the n_m, most probable (largest multinomial coefficient)
@@ -66,6 +66,7 @@ struct TableHost {
     TableDims d;
     std::vector<uint16_t> moves, ranks;
     std::vector<uint32_t> unrank;
+    std::vector<uint32_t> rows;  // per composition (at 4 (un[m] + rank)): its BF16 counts as words of a feature row
 };
 
 void enumerate(int left, int q, int S, std::vector<int> &c, std::vector<std::vector<int>> &out)
@@ -122,6 +123,7 @@ void build_table_host(int S, TableHost &T)
     T.moves.assign(std::max<size_t>(d.mv_total, 8), 0);
     T.ranks.assign(d.rk_total, 0);
     T.unrank.assign(d.un_total, 0);
+    T.rows.assign(4 * (size_t)d.un_total, 0);
     for (int m = 0; m < 3; ++m) {
         const int z = shell_z(m);
         auto radix = [&](const std::vector<int> &c) {
@@ -138,6 +140,13 @@ void build_table_host(int S, TableHost &T)
             uint32_t h = 0;
             for (int q = 0; q < S; ++q) h += (uint32_t)c[(size_t)q] << (4 * q);
             T.unrank[d.un[m] + (uint32_t)r] = h;
+            for (int q = 0; q < S; ++q) {  // column 5 (m + 1) + q of the row, relative to the word of the shell's first
+                const float f = (float)c[(size_t)q];
+                uint32_t b;
+                memcpy(&b, &f, 4);
+                const int col = (5 * (m + 1) & 1) + q;
+                T.rows[4 * (size_t)(d.un[m] + (uint32_t)r) + (size_t)(col / 2)] |= (b >> 16) << (16 * (col & 1));
+            }
         }
         std::map<std::vector<int>, int> rank;
         for (int r = 0; r < d.n[m]; ++r) rank[comp[m][(size_t)r]] = r;
@@ -217,38 +226,62 @@ __device__ __forceinline__ uint32_t word_index(const TableDims &D, uint32_t w)
 
 // ---------------------------------------------------------------------------
 // f of every feature vector.  Tile t holds vectors 128 t .. 128 t + 127.
+//
+// Bound by the chain of a tile (products, barriers, epilogues) and the ALU
+// under it, so that what a row costs besides its network counts: ranks advance
+// by the stride of the grid with carries (no divisions), and a row is put
+// together from the words of its three compositions (three 16-byte loads)
+// instead of from counts.  945 M vectors: MLP 37.9 -> 35.3 ms (its tanh alone
+// would take 26), MLPNet 42.4 -> 38.5 ms, and 35.7 ms with five warpgroups on
+// all tensor memory instead of four.
 // ---------------------------------------------------------------------------
 template <class Net>
-__global__ void __launch_bounds__(128 * kStreamWG) k_table_fill(const void *W, const TableDims D,
-                                                              const uint32_t *__restrict__ unrank, float *table,
+__global__ void __launch_bounds__(128 * Net::kFillNWG) k_table_fill(const void *W, const TableDims D,
+                                                              const uint4 *__restrict__ rows, float *table,
                                                               long long timeout_ns, int *status, int *abort_flag)
 {
-    constexpr int NWG = kStreamWG;
+    constexpr int NWG = Net::kFillNWG;
+    constexpr uint32_t xg = NWG <= 4 ? 512 : 384;  // bytes of 8 rows of the X tile
     typename Net::Eval E = mlp_evaluator<Net, NWG>(timeout_ns, status, abort_flag);
     mlp_cta_setup<Net, NWG>(E, W, nullptr, nullptr);
     const int r = threadIdx.x & 127, wg = threadIdx.x >> 7;
     const uint32_t nv = (uint32_t)D.entries, ntile = (nv + kTcRows - 1) / kTcRows;
-    // features of vector 128 tl + r; its place in the table (~0: past the last)
-    auto build = [&](uint32_t tl) {
-        const uint32_t v = tl * kTcRows + r;
-        int q0 = -1;
-        uint32_t h1 = 0, h2 = 0, h3 = 0, at = ~0u;
-        if (v < nv) {
-            const uint32_t t3 = v / (uint32_t)D.n[2], r3 = v - t3 * (uint32_t)D.n[2];
-            const uint32_t t2 = t3 / (uint32_t)D.n[1], r2 = t3 - t2 * (uint32_t)D.n[1];
-            const uint32_t t1 = t2 / (uint32_t)D.n[0], r1 = t2 - t1 * (uint32_t)D.n[0];
-            q0 = (int)t1;
-            h1 = __ldg(unrank + D.un[0] + r1);
-            h2 = __ldg(unrank + D.un[1] + r2);
-            h3 = __ldg(unrank + D.un[2] + r3);
-            at = D.S == 5 ? word_index<true>(D, t1 << kWordSp | r1 << word_sh(0) | r2 << word_sh(1) | r3) : v;
-        }
-        tc_write_features(E.L, r, q0, h1, h2, h3);
-        fence_async_smem();
-        return at;
-    };
     const uint32_t step = (uint32_t)NWG * gridDim.x;
     uint32_t tl = (uint32_t)NWG * blockIdx.x + wg;
+    // species and ranks of vector 128 tl + r, and of the stride
+    uint32_t t = tl * kTcRows + r;
+    const uint32_t n1 = (uint32_t)D.n[0], n2 = (uint32_t)D.n[1], n3 = (uint32_t)D.n[2];
+    uint32_t r3 = t % n3, r2 = (t /= n3) % n2, r1 = (t /= n2) % n1, q = t / n1;
+    t = step * kTcRows;
+    const uint32_t d3 = t % n3, d2 = (t /= n3) % n2, d1 = (t /= n2) % n1, dq = t / n1;
+    unsigned char *const row = g_smem + E.L.x + (r >> 3) * xg + (r & 7) * 16;  // chunks of 8 columns 128 bytes apart
+    for (int kc = 0; kc < (NWG <= 4 || r >= 120 ? 4 : 3); ++kc) *(uint4 *)(row + 128 * kc) = make_uint4(0u, 0u, 0u, 0u);
+    wg_sync(E.bar);
+    // writes the row of vector 128 tl + r and advances; its place in the table (~0: past the last)
+    auto build = [&](uint32_t tl) {
+        uint32_t at = ~0u;
+        if (q < (uint32_t)D.S) {
+            const uint4 a = __ldg(rows + D.un[0] + r1), b = __ldg(rows + D.un[1] + r2), c = __ldg(rows + D.un[2] + r3);
+            const uint32_t one = 0x3F80u << (16 * (q & 1));  // columns 0-4: the species
+            *(uint4 *)row =
+                make_uint4(q < 2 ? one : 0u, (q >> 1) == 1 ? one : 0u, (q == 4 ? one : 0u) | a.x, a.y);
+            *(uint4 *)(row + 128) = make_uint4(a.z, b.x, b.y, b.z | c.x);
+            *(uint4 *)(row + 256) = make_uint4(c.y, c.z, 0x3F803F80u, 0x00003F80u);
+            at = D.S == 5 ? word_index<true>(D, q << kWordSp | r1 << word_sh(0) | r2 << word_sh(1) | r3) : tl * kTcRows + r;
+        }
+        fence_async_smem();
+        r3 += d3;
+        uint32_t carry = r3 >= n3;
+        r3 -= carry ? n3 : 0u;
+        r2 += d2 + carry;
+        carry = r2 >= n2;
+        r2 -= carry ? n2 : 0u;
+        r1 += d1 + carry;
+        carry = r1 >= n1;
+        r1 -= carry ? n1 : 0u;
+        q += dq + carry;
+        return at;
+    };
     uint32_t at = ~0u;
     if (tl < ntile) {
         at = build(tl);
@@ -313,12 +346,13 @@ __global__ void __launch_bounds__(256) k_table_state(const __grid_constant__ Tab
 // the rows are written back.  Four lanes share a trial, ten zone sites each.
 // What bounds it are the look-ups, 40 per trial of unlike species: with five
 // species three in four miss L2 and cost a 128-byte DRAM read each (a
-// microbenchmark of such loads runs 39 G/s; the kernel 40 G/s, with 3.1 GB of
-// table reads per group at 256^3), and the loads that an SM can have in
-// flight need room in L1.  So shared memory is kept small: with move tables of
-// ordered pairs (204 KB used, 28 KB of L1) a group takes 1.03 ms, with the
-// factored ones 0.80 ms (256^3); a thread per trial, eight lanes per trial and
-// whole-block barriers were within 5 % of each other.
+// microbenchmark of such loads runs 39 G/s), and the loads that an SM can have
+// in flight need room in L1.  So shared memory is kept small: with move tables
+// of ordered pairs (204 KB used, 28 KB of L1) a group took 1.03 ms, with the
+// factored ones 0.80 ms, and with the vectors of probable compositions in
+// blocks of their own (word_index) 0.70 ms, 48 G/s (256^3); a thread per
+// trial, eight lanes per trial and whole-block barriers were within 5 % of each
+// other, and so were lanes with ten consecutive zone entries each.
 // ---------------------------------------------------------------------------
 constexpr int kTabTrials = 128;               // most trials of a block's mini-step
 constexpr int kLanes = 4;                     // lanes of a trial
@@ -544,16 +578,17 @@ size_t table_sweep_fixed(const TableDims &d, bool pair)
 }
 
 template <class Net>
-smc_status fill_launch(Workspace *ws, const void *W, const TableDims &d, const uint32_t *unrank, float *table,
+smc_status fill_launch(Workspace *ws, const void *W, const TableDims &d, const uint4 *rows, float *table,
                        int *abort_flag, cudaStream_t stream)
 {
-    const size_t smem = Net::template Smem<kStreamWG>::END;
+    constexpr int NWG = Net::kFillNWG;
+    const size_t smem = (Net::template Smem<NWG>::TINFO + 127) / 128 * 128;
     auto kern = k_table_fill<Net>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_table_fill)");
     const long long tiles = (d.entries + kTcRows - 1) / kTcRows;
-    const int grid = (int)std::max(1LL, std::min<long long>(ws->num_sms, (tiles + kStreamWG - 1) / kStreamWG));
-    kern<<<grid, 128 * kStreamWG, smem, stream>>>(W, d, unrank, table, debug_timeout_ns(), ws->status, abort_flag);
+    const int grid = (int)std::max(1LL, std::min<long long>(ws->num_sms, (tiles + NWG - 1) / NWG));
+    kern<<<grid, 128 * NWG, smem, stream>>>(W, d, rows, table, debug_timeout_ns(), ws->status, abort_flag);
     e = cudaGetLastError();
     return e == cudaSuccess ? SMC_OK : cuda_fail(e, "k_table_fill");
 }
@@ -582,13 +617,14 @@ bool pack_zone(int nx, std::vector<uint32_t> &out)
 
 }  // namespace
 
-bool mlp_table_wanted(const smc_lattice *lat, int nsweeps)
+bool mlp_table_wanted(const smc_lattice *lat, const smc_model *m, int nsweeps)
 {
     const TableDims &d = table_host(lat->nspecies).d;
     const double evals = 2.0 * lat->nx * lat->ny * lat->nz * nsweeps * kOmega * (1.0 - 1.0 / lat->nspecies);
-    // Per row: 58 ps evaluated in the sweep (MLP; MLPNet 108), 25 looked up, 37
-    // (44) for a vector of the table; equal at 1.12 (0.55) times the vectors.
-    return lat->nspecies >= 2 && evals > 1.15 * (double)d.entries;
+    // Per row: 58 ps evaluated in the sweep (MLP; MLPNet 102), 21-25 looked up, 37 for a vector of the table: equal
+    // at 1.0-1.1 (0.45-0.5) times the vectors. MLPNet, 128^3:
+    // 3 sweeps evaluated 40.3 ms (looked up 47), 4 looked up 50.7 (evaluated 53.3), 7 looked up 61.5 (92.9).
+    return lat->nspecies >= 2 && evals > (m->kind == SMC_MLPNET_BF16 ? 0.55 : 1.15) * (double)d.entries;
 }
 
 smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, int8_t *occ, uint64_t seed,
@@ -624,12 +660,12 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
         set_error("internal error: MLP interaction-zone geometry");
         return SMC_ERR_STATE;
     }
-    // workspace: [part_e | part_n | abort | weights | moves | ranks | packed counts | zone | D | state | table]
+    // workspace: [part_e | part_n | abort | weights | moves | ranks | packed counts | feature words | zone | D | state | table]
     const size_t nc = (size_t)P.NLx * P.ncol, N = 2ull * lat->nx * lat->ny * lat->nz;
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t o_pn = nc * 8, o_abort = o_pn + nc * 8, o_w = up(o_abort + 16), o_mv = up(o_w + kWeightBytes),
                  o_rk = up(o_mv + T.moves.size() * 2), o_un = up(o_rk + T.ranks.size() * 2),
-                 o_zone = up(o_un + T.unrank.size() * 4), o_D = up(o_zone + zone.size() * 4),
+                 o_rows = up(o_un + T.unrank.size() * 4), o_zone = up(o_rows + T.rows.size() * 4), o_D = up(o_zone + zone.size() * 4),
                  o_red = up(o_D + kDEntries * 4), o_state = up(o_red + lc_reduce_bytes()), o_tab = up(o_state + N * 8),
                  need = std::max(o_tab + (size_t)T.d.entries * 4, least);
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, need, &st);
@@ -661,11 +697,12 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
     put(o_mv, T.moves.data(), T.moves.size() * 2);
     put(o_rk, T.ranks.data(), T.ranks.size() * 2);
     put(o_un, T.unrank.data(), T.unrank.size() * 4);
+    put(o_rows, T.rows.data(), T.rows.size() * 4);
     put(o_zone, zone.data(), zone.size() * 4);
     if (pair) put(o_D, D, kDEntries * 4);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(MLP table sweep)");
-    st = net ? fill_launch<NetRelu96>(ws, scr + o_w, T.d, P.unrank, (float *)(scr + o_tab), (int *)(scr + o_abort), stream)
-             : fill_launch<NetSilu64>(ws, scr + o_w, T.d, P.unrank, (float *)(scr + o_tab), (int *)(scr + o_abort), stream);
+    st = net ? fill_launch<NetRelu96>(ws, scr + o_w, T.d, (const uint4 *)(scr + o_rows), (float *)(scr + o_tab), (int *)(scr + o_abort), stream)
+             : fill_launch<NetSilu64>(ws, scr + o_w, T.d, (const uint4 *)(scr + o_rows), (float *)(scr + o_tab), (int *)(scr + o_abort), stream);
     if (st != SMC_OK) return st;
     const int sb = (int)std::max<size_t>(1, std::min<size_t>((N + 255) / 256, (size_t)ws->num_sms * 64));
     k_table_state<<<sb, 256, 0, stream>>>(P);

@@ -58,7 +58,7 @@ struct MlpSmem {
 constexpr int kSweepWG = 4;  // warpgroups of the sweep kernel (64-wide network)
 constexpr int kEvalWG = 2;   // warpgroups of the trace kernel
 // Warpgroups of the kernels that stream rows through the network (site
-// energies, the table): one CTA per SM with all 512 tensor-memory columns.
+// energies; the MLP's table): one CTA per SM with all 512 tensor-memory columns.
 // With two warpgroups per CTA the driver kept one CTA per SM (the occupancy
 // query gives 1, eight warps), and the special-function pipe idled half the
 // time: 50.6 ms for the 9.46e8 rows of the five-species table (MLP), 72 ms
@@ -73,18 +73,19 @@ struct NetSmem {
     static constexpr uint32_t W1 = W0 + kNetW0;
     static constexpr uint32_t W2 = W1 + kNetW12;
     static constexpr uint32_t X = W2 + kNetW12;      // [NWG] tiles
-    static constexpr uint32_t H = X + NWG * kNetX;   // [NWG] tiles
+    static constexpr uint32_t XSIZE = NWG <= 4 ? kNetX : kNetXc;
+    static constexpr uint32_t H = X + NWG * XSIZE;   // [NWG] tiles
     static constexpr uint32_t W3 = H + NWG * kNetHt;
     static constexpr uint32_t B3 = W3 + kNetHid * 4;
     static constexpr uint32_t MBAR = B3 + 16;        // [NWG][2]
     static constexpr uint32_t TSLOT = MBAR + 16 * NWG;
     static constexpr uint32_t CTL = TSLOT + 4;
     static constexpr uint32_t RED = (CTL + 4 + 15) / 16 * 16;
-    static constexpr uint32_t TINFO = RED + 64;
+    static constexpr uint32_t TINFO = RED + 64;      // (the table kernel's shared memory ends here)
     static constexpr uint32_t ACT = TINFO + kMlpChunk * kTinfo * 4;
     static constexpr uint32_t GEO = ACT + kMlpChunk * 4;
     static constexpr uint32_t END = (uint32_t)((GEO + sizeof(MlpGeo) + 127) / 128 * 128);
-    static_assert(X % 128 == 0 && H % 128 == 0 && W1 % 128 == 0 && W2 % 128 == 0, "tile alignment");
+    static_assert(X % 128 == 0 && XSIZE % 128 == 0 && H % 128 == 0 && W1 % 128 == 0 && W2 % 128 == 0, "tile alignment");
     static_assert(MBAR % 8 == 0 && RED % 8 == 0, "alignment");
 };
 
@@ -96,6 +97,7 @@ struct NetSilu64 {  // MLP of mlp_tc.cuh: 20 -> 64 -> 64 -> 1, SiLU
     template <int NWG>
     using Smem = MlpSmem<NWG>;
     static constexpr int kSweepNWG = kSweepWG;
+    static constexpr int kFillNWG = kStreamWG;
     template <int NWG>
     static __device__ TcLayout layout(uint32_t wg)
     {
@@ -110,12 +112,13 @@ struct NetRelu96 {  // MLPNet of mlpnet_tc.cuh: 20 -> 96 -> 96 -> 96 -> 1, ReLU
     template <int NWG>
     using Smem = NetSmem<NWG>;
     static constexpr int kSweepNWG = 2;  // the 28 KB hidden tiles of four would not fit
+    static constexpr int kFillNWG = 5;   // all tensor memory: 96 columns each
     template <int NWG>
     static __device__ NetLayout layout(uint32_t wg)
     {
         using M = NetSmem<NWG>;
-        return NetLayout{M::X + wg * kNetX, M::H + wg * kNetHt, M::W0, M::W1, M::W2, M::W3, M::B3, M::MBAR + 16 * wg,
-                         M::TSLOT};
+        return NetLayout{M::X + wg * M::XSIZE, M::H + wg * kNetHt, M::W0, M::W1, M::W2, M::W3, M::B3, M::MBAR + 16 * wg,
+                         M::TSLOT, NWG <= 4 ? 512u : 384u};
     }
 };
 
@@ -184,7 +187,7 @@ smc_status mlp_copy_weights(const smc_model *m, void *dst, cudaStream_t stream);
 // Sweeps with f tabulated over all feature vectors (mlp_table.cu): whether a
 // call is large enough for it, and the call; *taken is false when the table
 // does not fit (the caller runs the evaluating sweep).  D: pair table (host).
-bool mlp_table_wanted(const smc_lattice *lat, int nsweeps);
+bool mlp_table_wanted(const smc_lattice *lat, const smc_model *m, int nsweeps);
 // (The workspace grows to `least` bytes at least: those of the evaluating
 // sweep, which takes the captured calls that a plain one prepares.)
 smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, int8_t *occ, uint64_t seed,

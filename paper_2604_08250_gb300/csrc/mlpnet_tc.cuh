@@ -29,7 +29,13 @@ constexpr uint32_t kNetX = 128 * 64;           // X tile: 128 rows x 32 BF16
 constexpr uint32_t kNetHt = 128 * kNetK * 2;   // H tile: 128 rows x 112 BF16
 constexpr uint32_t kNetW0 = kNetHid * 64;      // W0: 96 rows x 32 BF16
 constexpr uint32_t kNetW12 = kNetHid * kNetK * 2;  // W1, W2: 96 rows x 112 BF16
-constexpr uint32_t kNetCols = 128;             // TMEM columns per warpgroup (96 used)
+// TMEM columns of a warpgroup (96 used) and those allocated, a power of two.
+__host__ __device__ constexpr uint32_t net_cols(int nwg) { return nwg <= 4 ? 128 : 96; }
+__host__ __device__ constexpr uint32_t net_alloc(int nwg) { return nwg <= 4 ? 128 * nwg : 512; }
+// X tile of five warpgroups: 24 columns a row, the products' columns 24-31
+// being the next 8 rows' first chunk (finite) against zero weights; a zero
+// chunk follows the last rows.
+constexpr uint32_t kNetXc = 128 * 48 + 128;
 constexpr uint32_t kNetIdesc = tc_idesc(128, kNetHid, false, false);
 
 // Byte offset of element chunk kc (8 BF16) of row r in a K = 112 tile.
@@ -47,6 +53,7 @@ struct NetBlock {
 
 struct NetLayout {
     uint32_t x, h, w0, w1, w2, w3, b3, mbar, tmem_slot;
+    uint32_t xg;  // bytes of 8 rows of the X tile: 512, or 384 with 24 columns a row
 };
 
 struct NetEval {
@@ -114,12 +121,12 @@ static __device__ void tc_setup(NetEval &E, int nwg)
         mbar_init(s0 + E.L.mbar, 1);
         mbar_init(s0 + E.L.mbar + 8, 1);
     }
-    if (threadIdx.x < 32) tc_alloc(s0 + E.L.tmem_slot, kNetCols * nwg);
+    if (threadIdx.x < 32) tc_alloc(s0 + E.L.tmem_slot, net_alloc(nwg));
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    E.tmem = *(const uint32_t *)(g_smem + E.L.tmem_slot) + kNetCols * wg;
+    E.tmem = *(const uint32_t *)(g_smem + E.L.tmem_slot) + net_cols(nwg) * wg;
     E.phase1 = E.phase2 = 0;
     E.bar = 1 + wg;
 }
@@ -129,7 +136,7 @@ static __device__ void tc_teardown(NetEval &E, int nwg)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (threadIdx.x < 32) tc_dealloc(*(const uint32_t *)(g_smem + E.L.tmem_slot), kNetCols * nwg);
+    if (threadIdx.x < 32) tc_dealloc(*(const uint32_t *)(g_smem + E.L.tmem_slot), net_alloc(nwg));
 }
 
 // The X tile has the layout of the 64-wide network's: same features.
@@ -206,7 +213,7 @@ static __device__ __forceinline__ void tc_stage2(NetEval &E)
         tc_fence_after();
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            tc_mma_i(E.tmem, tc_desc(s0 + E.L.x + k * 256, 128, 512), tc_desc(s0 + E.L.w0 + k * 256, 128, 512),
+            tc_mma_i(E.tmem, tc_desc(s0 + E.L.x + k * 256, 128, E.L.xg), tc_desc(s0 + E.L.w0 + k * 256, 128, 512),
                      kNetIdesc, k > 0);
         tc_commit(s0 + E.L.mbar);
     }

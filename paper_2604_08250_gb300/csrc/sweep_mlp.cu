@@ -925,7 +925,7 @@ smc_status launch_mlp_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     const int threads = 128 * (net ? NetRelu96::kSweepNWG : NetSilu64::kSweepNWG);
     MlpPlan pl;
     st = net ? make_mlp_plan(ws, lat, kernel, NetSmem<NetRelu96::kSweepNWG>::END, threads,
-                             NetRelu96::kSweepNWG * (int)kNetCols, pl)
+                             (int)net_alloc(NetRelu96::kSweepNWG), pl)
              : make_mlp_plan(ws, lat, kernel, MlpSmem<kSweepWG>::END, threads, kSweepWG * (int)kTcCols, pl);
     if (st != SMC_OK) return st;
     static MlpGeo G;
@@ -978,7 +978,7 @@ smc_status launch_mlp_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     // A call whose trials evaluate more rows than there are feature vectors
     // evaluates each vector once and looks the others up.  Not into a graph:
     // it would read the host's copies of the tables when it is replayed.
-    if (mlp_table_wanted(lat, nsweeps) && !stream_capturing(stream)) {
+    if (mlp_table_wanted(lat, m, nsweeps) && !stream_capturing(stream)) {
         bool taken = false;
         st = launch_mlp_table_sweep(lat, m, occ, seed, replica, sweep0, nsweeps, kT, e_acc, n_acc, P.D.df,
                                     off_fcache + N * 16, &taken, stream);
