@@ -720,7 +720,8 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
     const int NLy = ny / 4, NLz = nz / 4, nsh = pt.nsh;
     // row pitch: a multiple of 128 bytes when the windows fit with it, so that
     // the same x of every row falls in the same bank (the lanes' partner rows
-    // differ per lane; their x do not), else the 16-byte halos only
+    // differ per lane; their x do not), else the 16-byte halos only, to a
+    // multiple of 16
     int rowB = (nx + 32 + 127) / 128 * 128;
     const void *kern = pick_resident<IS_INT>(pt.nsh, pt.sw);
     cudaFuncAttributes fa;
@@ -908,7 +909,7 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
         return (size_t)kQRows * pt.rw * 4 + 64 + (size_t)2 * rp.Wy * rp.Wz * pitch +
                ((size_t)rp.blob * 4 + 15) / 16 * 16 + (size_t)nc * nk * 512;
     };
-    if (smem_of(rowB) > dyn_max) rowB = nx + 32;
+    if (smem_of(rowB) > dyn_max) rowB = (nx + 32 + 15) / 16 * 16;  // (the exchange moves 8 and 16 bytes)
     rp.rowB = rowB;
     const size_t smem = smem_of(rowB);
     if (smem > dyn_max) return SMC_OK;
