@@ -43,6 +43,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <set>
 #include <vector>
@@ -61,7 +62,15 @@ namespace {
 // [17] row pitch, [18] offset of the replica's lattice copy (bytes),
 // [19] offset of its version slots (words), [20] its version slots.
 constexpr int kResDesc = 24;
-constexpr int kResCols = 8;  // compute warps per CTA (columns per block at most)
+// Compute warps per CTA (columns per block at most): 8, or 16 where replicas
+// that share launches take fewer waves so (res_cols) and for a lattice that
+// fits the SMs only in such blocks.
+constexpr int kResCols = 8, kResColsWide = 16;
+// Exchange warps: with three a wide CTA has 20 warps, five per scheduler, and
+// its threads 96 registers (21 warps: 80, and spills).
+__host__ __device__ constexpr int res_xw(int nc) { return nc == kResCols ? 4 : 3; }
+constexpr int kResWideRow = 96;       // cells of the longest rows at a pitch of 128 bytes: 135 KB a wide block
+constexpr double kResWideCost = 1.35;  // a group of wide blocks over one of the others
 
 // The exchange warps prepare group g once the compute warps finished group
 // g - kAhead - 1, so while groups g - kAhead .. g - 1 may still wait for
@@ -331,8 +340,8 @@ __device__ bool res_fetch_versions(const SweepParams &P, const unsigned long lon
 // compile time (0: read from the descriptor), so that the trial's row offsets
 // are immediates.  Those kernels (two shells, one species word) also take
 // the replicated pair table (res_xb_table).
-template <bool IS_INT, int NSH, int SW, int RB, int WY>
-__global__ void __launch_bounds__(416, 1) k_sweep_resident(const __grid_constant__ SweepParams P)
+template <bool IS_INT, int NSH, int SW, int RB, int WY, int NC = kResCols>
+__global__ void __launch_bounds__((NC + res_xw(NC) + 1) * 32, 1) k_sweep_resident(const __grid_constant__ SweepParams P)
 {
     constexpr bool XB = RB != 0 && WY != 0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
@@ -693,29 +702,84 @@ int res_slot_of(const int *dd, int r, int ny, int nz, int Wy, int Wz)
     return (s * Wz + zz) * Wy + yy;
 }
 
-template <bool IS_INT>
-const void *pick_resident(int nsh, int sw)
+template <bool IS_INT, int NC>
+const void *pick_resident_nc(int nsh, int sw)
 {
     if (nsh >= 3)
-        return sw == 2 ? (const void *)k_sweep_resident<IS_INT, 3, 2, 0, 0>
-                       : (const void *)k_sweep_resident<IS_INT, 3, 1, 0, 0>;
-    return sw == 2 ? (const void *)k_sweep_resident<IS_INT, 2, 2, 0, 0> : (const void *)k_sweep_resident<IS_INT, 2, 1, 0, 0>;
+        return sw == 2 ? (const void *)k_sweep_resident<IS_INT, 3, 2, 0, 0, NC>
+                       : (const void *)k_sweep_resident<IS_INT, 3, 1, 0, 0, NC>;
+    return sw == 2 ? (const void *)k_sweep_resident<IS_INT, 2, 2, 0, 0, NC>
+                   : (const void *)k_sweep_resident<IS_INT, 2, 1, 0, 0, NC>;
 }
-// the specialisation for blocks of 2 x 4 columns on 128-cell rows (pitch 256
-// bytes, 15 window rows per y), when every block of a launch has them
 template <bool IS_INT>
-const void *pick_resident_fixed(int nsh, int sw, int rowB, int Wy)
+const void *pick_resident(int nsh, int sw, int nc)
 {
-    if (nsh == 2 && sw == 1 && rowB == 256 && Wy == 15) return (const void *)k_sweep_resident<IS_INT, 2, 1, 256, 15>;
+    return nc == kResCols ? pick_resident_nc<IS_INT, kResCols>(nsh, sw) : pick_resident_nc<IS_INT, kResColsWide>(nsh, sw);
+}
+// the specialisations for blocks of 2 x 4 columns on 128-cell rows (pitch 256
+// bytes, 15 window rows per y) and for wide blocks on rows of up to 96 cells
+// (128, 23), when every block of a launch has them
+template <bool IS_INT>
+const void *pick_resident_fixed(int nsh, int sw, int nc, int rowB, int Wy)
+{
+    if (nsh != 2 || sw != 1) return nullptr;
+    if (nc == kResCols && rowB == 256 && Wy == 15) return (const void *)k_sweep_resident<IS_INT, 2, 1, 256, 15>;
+    if (nc == kResColsWide && rowB == 128 && Wy == 23)
+        return (const void *)k_sweep_resident<IS_INT, 2, 1, 128, 23, kResColsWide>;
     return nullptr;
+}
+
+// Window rows along y of a block by columns wide; wide blocks all have those of
+// four columns, so that their kernel knows the number.
+constexpr int res_wy(int by, int ncols) { return ncols == kResCols ? 4 * by + 7 : 23; }
+
+// Columns per block (by x bz) of a lattice, at most ncols, at most one block
+// per SM and at least 3 blocks per axis: the fewest columns per block (the
+// shortest group; with few_blocks, for replicas sharing a launch, the most, or
+// of wide blocks the fewest blocks), then the fewest rows held.  A tuned tile
+// shape (tile_y, tile_z) selects the block shape.  False: none.
+bool res_shape(const smc_lattice &lat, int num_sms, bool few_blocks, int ncols, int &by_out, int &bz_out)
+{
+    const int shapes[][2] = {{1, 1}, {1, 2}, {2, 1}, {2, 2}, {1, 4}, {4, 1}, {2, 3}, {3, 2}, {2, 4}, {4, 2}, {1, 8}, {8, 1},
+                             {3, 3}, {3, 4}, {4, 3}, {4, 4}};
+    const int NLy = lat.ny / 4, NLz = lat.nz / 4;
+    const Tuning tu = current_tuning();
+    int best = -1, best_nc = 1 << 30, best_rows = 1 << 30, best_blocks = 1 << 30;
+    for (int i = 0; i < (int)(sizeof shapes / sizeof shapes[0]); ++i) {
+        const int by = shapes[i][0], bz = shapes[i][1];
+        if (by * bz > ncols || (ncols > kResCols && by > 4)) continue;
+        if (tu.tile_y > 0 && tu.tile_z > 0 && (by != tu.tile_y || bz != tu.tile_z)) continue;
+        const int NBy = (NLy + by - 1) / by, NBz = (NLz + bz - 1) / bz;
+        if (NBy < 3 || NBz < 3 || NBy * NBz > num_sms) continue;
+        const int Wy = res_wy(by, ncols), Wz = 4 * bz + 7;
+        if (Wy >= lat.ny || Wz >= lat.nz) continue;
+        const int nrows = 2 * Wy * Wz, nc = by * bz, nb = NBy * NBz;
+        bool better;
+        if (ncols > kResCols)
+            better = nb < best_blocks || (nb == best_blocks && nrows < best_rows);
+        else
+            better = (few_blocks ? (best < 0 || nc > best_nc) : nc < best_nc) || (nc == best_nc && nrows < best_rows);
+        if (better) {
+            best = i;
+            best_nc = nc;
+            best_rows = nrows;
+            best_blocks = nb;
+        }
+    }
+    if (best < 0) return false;
+    by_out = shapes[best][0];
+    bz_out = shapes[best][1];
+    return true;
 }
 
 // Builds the plan for one lattice, or leaves ok = 0 when the lattice does not
 // fit (the streaming kernel then runs).
 template <bool IS_INT>
-smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace *ws, bool few_blocks, ResPlan &rp)
+smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace *ws, bool few_blocks, int ncols,
+                          ResPlan &rp)
 {
     rp = ResPlan();
+    rp.nxw = res_xw(ncols);
     const int nx = lat.nx, ny = lat.ny, nz = lat.nz;
     const int NLy = ny / 4, NLz = nz / 4, nsh = pt.nsh;
     // row pitch: a multiple of 128 bytes when the windows fit with it, so that
@@ -723,43 +787,20 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
     // differ per lane; their x do not), else the 16-byte halos only, to a
     // multiple of 16
     int rowB = (nx + 32 + 127) / 128 * 128;
-    const void *kern = pick_resident<IS_INT>(pt.nsh, pt.sw);
+    const void *kern = pick_resident<IS_INT>(pt.nsh, pt.sw, ncols);
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, kern);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes");
     const size_t dyn_max = ws->smem_optin - fa.sharedSizeBytes;
-    // block shapes with at most 8 columns, at most one CTA per SM and at
-    // least 3 blocks per axis; the fewest columns per block (the shortest
-    // group; with few_blocks, for replicas sharing a launch, the most), then
-    // the fewest rows held.  A tuned tile shape (tile_y, tile_z) selects the
-    // block shape.
-    const int shapes[][2] = {{1, 1}, {1, 2}, {2, 1}, {2, 2}, {1, 4}, {4, 1}, {2, 3}, {3, 2}, {2, 4}, {4, 2}, {1, 8}, {8, 1}};
-    const Tuning tu = current_tuning();
-    int best = -1, best_nc = 1 << 30, best_rows = 1 << 30;
-    for (int i = 0; i < (int)(sizeof shapes / sizeof shapes[0]); ++i) {
-        const int by = shapes[i][0], bz = shapes[i][1];
-        if (tu.tile_y > 0 && tu.tile_z > 0 && (by != tu.tile_y || bz != tu.tile_z)) continue;
-        const int NBy = (NLy + by - 1) / by, NBz = (NLz + bz - 1) / bz;
-        if (NBy < 3 || NBz < 3 || NBy * NBz > ws->num_sms) continue;
-        const int Wy = 4 * by + 7, Wz = 4 * bz + 7;
-        if (Wy >= ny || Wz >= nz) continue;
-        const int nrows = 2 * Wy * Wz, nc = by * bz;
-        const bool better_nc = few_blocks ? (best < 0 || nc > best_nc) : nc < best_nc;
-        if (better_nc || (nc == best_nc && nrows < best_rows)) {
-            best = i;
-            best_nc = nc;
-            best_rows = nrows;
-        }
-    }
-    if (best < 0 || nx % 4 != 0) return SMC_OK;
-    const int by = shapes[best][0], bz = shapes[best][1];
+    int by = 0, bz = 0;
+    if (nx % 4 != 0 || !res_shape(lat, ws->num_sms, few_blocks, ncols, by, bz)) return SMC_OK;
     rp.by = by;
     rp.bz = bz;
     rp.NBy = (NLy + by - 1) / by;
     rp.NBz = (NLz + bz - 1) / bz;
     rp.nblocks = rp.NBy * rp.NBz;
     rp.nc = by * bz;
-    rp.Wy = 4 * by + 7;
+    rp.Wy = res_wy(by, ncols);
     rp.Wz = 4 * bz + 7;
     rp.rowB = rowB;
     const int nrows_lat = 2 * ny * nz;
@@ -785,7 +826,7 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
     };
     rp.desc.assign((size_t)rp.nblocks * kResDesc, 0);
     rp.lists.clear();
-    const int nc = kResCols;  // compute warps of the kernel (some idle for smaller blocks)
+    const int nc = ncols;  // compute warps of the kernel (some idle for smaller blocks)
     std::vector<int> vslot((size_t)32 * nrows_lat, -1);  // (group of the write, row) -> version slot
     int nver = 0;
     struct Blk {
@@ -920,7 +961,7 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_max);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (kResCols + rp.nxw + 1) * 32, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (ncols + rp.nxw + 1) * 32, smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     if (per_sm < 1 || rp.nblocks > per_sm * ws->num_sms) return SMC_OK;
     rp.per_sm = per_sm;
@@ -966,6 +1007,7 @@ struct ResWave {
 
 struct ResMulti {
     bool ok = false;
+    int ncols = kResCols;  // compute warps per CTA
     const void *kernel = nullptr;
     std::vector<ResPlan> rp;
     std::vector<ResWave> waves;
@@ -978,13 +1020,45 @@ void free_waves(ResMulti &mp)
     mp.waves.clear();
 }
 
+// Compute warps per CTA for R replicas.  A wave's time is its groups', 2.77 us
+// each with 8 warps, 3.6 us with 16 (bound by issue then, where 8 leave the
+// schedulers waiting for each other's rows half of the time), so wide blocks
+// are taken when they save enough waves.  64 cubes of 32-96 cells, 20 sweeps:
+// 16 waves in 28.4 ms, or 9 wide ones in 20.7 ms (21.3 ms without the kernel
+// that knows pitch and window).
+int res_cols(int R, const smc_lattice *lats, int num_sms)
+{
+    const Tuning tu = current_tuning();
+    if (R < 2 || (tu.tile_y > 0 && tu.tile_z > 0)) return kResCols;
+    int waves[2] = {0, 0};
+    for (int wide = 0; wide < 2; ++wide) {
+        std::vector<int> nb, bins;
+        for (int r = 0; r < R; ++r) {
+            int by = 0, bz = 0;
+            if (!res_shape(lats[r], num_sms, true, wide ? kResColsWide : kResCols, by, bz)) return kResCols;
+            if (wide && lats[r].nx > kResWideRow) return kResCols;
+            nb.push_back(((lats[r].ny / 4 + by - 1) / by) * ((lats[r].nz / 4 + bz - 1) / bz));
+        }
+        std::sort(nb.begin(), nb.end(), std::greater<int>());
+        for (int n : nb) {  // first fit, as the waves are filled
+            size_t i = 0;
+            while (i < bins.size() && bins[i] + n > num_sms) ++i;
+            if (i == bins.size()) bins.push_back(0);
+            bins[i] += n;
+        }
+        waves[wide] = (int)bins.size();
+    }
+    return waves[1] * kResWideCost < waves[0] ? kResColsWide : kResCols;
+}
+
 template <bool IS_INT>
-smc_status build_res_multi(int R, const smc_lattice *lats, const PairTable &pt, Workspace *ws, ResMulti &mp)
+smc_status build_res_multi(int R, const smc_lattice *lats, const PairTable &pt, Workspace *ws, int ncols, ResMulti &mp)
 {
     mp = ResMulti();
+    mp.ncols = ncols;
     for (int r = 0; r < R; ++r) {
         ResPlan rp;
-        const smc_status st = build_res_plan<IS_INT>(lats[r], pt, ws, R > 1, rp);
+        const smc_status st = build_res_plan<IS_INT>(lats[r], pt, ws, R > 1, ncols, rp);
         if (st != SMC_OK) return st;
         if (!rp.ok) return SMC_OK;
         mp.kernel = rp.kernel;
@@ -992,7 +1066,7 @@ smc_status build_res_multi(int R, const smc_lattice *lats, const PairTable &pt, 
     }
     bool same = true;
     for (const auto &rp : mp.rp) same = same && rp.rowB == mp.rp[0].rowB && rp.Wy == mp.rp[0].Wy;
-    const void *fixed = same ? pick_resident_fixed<IS_INT>(pt.nsh, pt.sw, mp.rp[0].rowB, mp.rp[0].Wy) : nullptr;
+    const void *fixed = same ? pick_resident_fixed<IS_INT>(pt.nsh, pt.sw, ncols, mp.rp[0].rowB, mp.rp[0].Wy) : nullptr;
     cudaFuncAttributes fa;
     cudaError_t e;
     if (fixed) {
@@ -1016,7 +1090,7 @@ smc_status build_res_multi(int R, const smc_lattice *lats, const PairTable &pt, 
         }
         const size_t smax = base + pad(maxblob);
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fixed, (kResCols + mp.rp[0].nxw + 1) * 32, smax);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fixed, (ncols + mp.rp[0].nxw + 1) * 32, smax);
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
         if (smax <= fdyn && per_sm >= need_sm) {
             mp.kernel = fixed;
@@ -1133,7 +1207,18 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
         free_waves(plan_cached);
         key_cached.clear();
         ResMulti mp;
-        st = is_int ? build_res_multi<true>(R, lats, pt, ws, mp) : build_res_multi<false>(R, lats, pt, ws, mp);
+        // Wide blocks that do not fit after all: the others.  One lattice with more columns than 152 blocks of 8 hold
+        // (up to 2,432 short rows): wide ones.  20 sweeps, streaming / resident: 64 x 160 x 160 5.4 / 2.3 ms, three
+        // shells of eight species 6.2 / 3.6 ms, 100 x 160 x 160 8.3 / 2.8 ms, 128 x 160 x 160 3.3 / 2.8 ms,
+        // 140 x 144 x 144 11.4 / 4.2 ms; 160-cell rows no longer fit.
+        const int first = res_cols(R, lats, ws->num_sms);
+        const int second = first != kResCols ? kResCols : (R == 1 ? kResColsWide : 0);
+        for (int ncols : {first, second}) {
+            if (!ncols) break;
+            free_waves(mp);
+            st = is_int ? build_res_multi<true>(R, lats, pt, ws, ncols, mp) : build_res_multi<false>(R, lats, pt, ws, ncols, mp);
+            if (st != SMC_OK || mp.ok) break;
+        }
         plan_cached = std::move(mp);
         if (st != SMC_OK) {
             free_waves(plan_cached);
@@ -1179,7 +1264,7 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
         exmax = std::max(exmax, w.exch_bytes);
         vwmax = std::max(vwmax, w.ver_words);
     }
-    const size_t np = nbmax * kResCols;
+    const size_t np = nbmax * (size_t)mp.ncols;
     const size_t off_flags = 0, off_pe = ((nbmax * 4 + 15) / 16) * 16, off_pn = off_pe + np * 8;
     const size_t off_misc = off_pn + np * 8, off_tab = off_misc + 16;
     const size_t off_exch = off_tab + ((tabs.size() * 4 + 255) / 256) * 256;
@@ -1267,7 +1352,7 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
             e = cudaGetLastError();
             if (e != cudaSuccess) return cuda_fail(e, "k_occ_to_exch");
             void *args[] = {(void *)&P};
-            e = cudaLaunchCooperativeKernel(mp.kernel, dim3(w.nblocks), dim3((kResCols + P.rxw + 1) * 32), args,
+            e = cudaLaunchCooperativeKernel(mp.kernel, dim3(w.nblocks), dim3((mp.ncols + P.rxw + 1) * 32), args,
                                             w.smem, stream);
             if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchCooperativeKernel(resident sweep)");
         }

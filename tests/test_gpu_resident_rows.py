@@ -58,3 +58,19 @@ def _same(smc, dims, kind, S, nsh):
 def test_rows_of_half_chunks_at_the_short_pitch(smc):
     """228 cells: windows too large for a pitch of 128-byte multiples, rows no multiple of 8 bytes."""
     _same(smc, [(228, 128, 136)], "f32", 5, 2)
+
+
+@pytest.mark.parametrize("dims,kind,S,nsh", [((12, 144, 140), "f32", 5, 2), ((64, 144, 140), "f32", 8, 3),
+                                             ((96, 140, 144), "int", 4, 2), ((100, 144, 140), "f32", 5, 2),
+                                             ((140, 140, 144), "f32", 3, 1), ((36, 196, 196), "int", 8, 2),
+                                             ((128, 144, 140), "f32", 5, 2), ((160, 144, 140), "f32", 5, 2)])
+def test_wide_blocks(smc, dims, kind, S, nsh):
+    """More columns than 152 blocks of eight hold: blocks of up to sixteen (the last box fits in neither)."""
+    _same(smc, [dims], kind, S, nsh)
+
+
+@pytest.mark.parametrize("edges,kind,nsh", [([64] * 12, "f32", 2), ([96, 84, 64, 52, 36, 32] * 4, "int", 2),
+                                            ([80] * 9 + [40], "f32", 3), ([96] * 6 + [100], "f32", 2)])
+def test_wide_blocks_of_replicas(smc, edges, kind, nsh):
+    """Replicas that take fewer launches in wide blocks, with odd lattices among them; and, last, a row too long."""
+    _same(smc, [(e, e, e) for e in edges], kind, 5, nsh)
