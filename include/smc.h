@@ -164,19 +164,23 @@ smc_status smc_init_lattice(const smc_lattice *lat, const int64_t *counts, uint6
  * per-shell species counts, 16 N bytes) the same way; they need every axis
  * a multiple of 4 cells and >= 8, nx <= 1024.  A call that would evaluate
  * more rows than there are feature vectors (9.5e8 for five species: about
- * one sweep of 256^3) evaluates every vector once and looks the others up
- * (8 N bytes and 4 bytes per vector of workspace; without room for them it
- * runs as a smaller call does), with the same results bit for bit.  qSRO models keep each site's
- * own-species count per shell (N bytes for 1-2 shells, 2 N for 3), built at
- * the start of every call and updated by accepted swaps; a trial's dE comes
+ * one sweep of 256^3; MLPNet half as many) evaluates every vector once and
+ * looks the others up (8 N bytes and 4 bytes per vector of workspace; without
+ * room for them, and into a CUDA graph, it runs as a smaller call does), with
+ * the same results bit for bit.  qSRO models keep each site's own-species
+ * count per shell (N bytes for 1-2 shells, 2 N for 3), built at the start of
+ * every call and updated by accepted swaps (boxes of up to 1024 cells per row
+ * run the four mini-steps of a group in one launch); a trial's dE comes
  * from the species of a, b and the sites within the model's shells of
  * either, and from those sites' counts, in FP32 (C left out, where it
  * cancels), within 1e-5 eV of FP64.  They need every axis a multiple of 4
  * cells and >= 8.
  * Pair models on lattices with every axis a multiple of 4 and >= 8 cells
- * whose rows fit the SMs' shared memory (128^3 and below) keep the lattice
- * there for the whole call (one cooperative launch per call, row versions
- * exchanged between CTAs through L2); larger lattices stream their rows from
+ * whose rows fit the SMs' shared memory (128^3 and below, and up to 2,432
+ * rows of link cells of at most 140 cells) keep the lattice there for the
+ * whole call (one cooperative launch per call, row versions exchanged between
+ * CTAs through L2); boxes of few link cells run in one CTA each; larger
+ * lattices stream their rows from
  * device memory (rows of 128, 256 or 512 cells with a two-shell model of at
  * most 5 species and a 16-byte aligned occ: two groups of mini-steps per
  * staging of a column's rows).  All give the same trajectory bit for bit.

@@ -1204,6 +1204,7 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
     std::vector<long long> key = {R, pt.nsh, pt.sw, is_int, ws->device, ws->num_sms, tu.tile_y, tu.tile_z};
     for (int r = 0; r < R; ++r) key.insert(key.end(), {lats[r].nx, lats[r].ny, lats[r].nz});
     if (key != key_cached) {
+        if (stream_capturing(stream)) return SMC_ERR_UNSUPPORTED;  // a plan's lists cannot be allocated into a graph
         free_waves(plan_cached);
         key_cached.clear();
         ResMulti mp;
@@ -1217,6 +1218,12 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
             if (!ncols) break;
             free_waves(mp);
             st = is_int ? build_res_multi<true>(R, lats, pt, ws, ncols, mp) : build_res_multi<false>(R, lats, pt, ws, ncols, mp);
+            if (R == 1 && ncols == kResColsWide && st != SMC_OK) {  // no room for the lists: the streaming kernels
+                cudaGetLastError();
+                free_waves(mp);
+                mp.ok = false;
+                st = SMC_OK;
+            }
             if (st != SMC_OK || mp.ok) break;
         }
         plan_cached = std::move(mp);
@@ -1270,6 +1277,10 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
     const size_t off_exch = off_tab + ((tabs.size() * 4 + 255) / 256) * 256;
     const size_t off_ver = off_exch + exmax;
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, off_ver + vwmax * 8, &st);
+    if (!scr && R == 1 && mp.ncols == kResColsWide) {  // the streaming kernels need less
+        cudaGetLastError();
+        return SMC_ERR_UNSUPPORTED;
+    }
     if (!scr) return st;
     cudaError_t e = cudaSuccess;
     if (!tabs.empty()) {

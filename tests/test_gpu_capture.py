@@ -61,3 +61,21 @@ def test_energy(smc, dims):
     torch.cuda.synchronize()
     smc.check()
     assert e.item() == plain.item()
+
+
+@pytest.mark.parametrize("warm", [False, True])
+def test_pair_sweep_of_many_short_rows(smc, warm):
+    """A lattice that only wide resident blocks hold: captured without a plan it streams, with one it stays resident."""
+    lat, occ = _start(smc, (16, 144, 140), 5, 6)
+    model = smc.Model(smc.PAIR_F32, 2, inputs.pair_f32_coeffs(9, 2, 5))
+    kT = [0.08, 0.07]
+    plain, again = occ.clone(), occ.clone()
+    smc.sweep(lat, model, plain, 5, 0, 2, kT)
+    if not warm:  # another lattice's plan takes the place of this one's
+        other, oocc = _start(smc, (64, 64, 64), 5, 7)
+        smc.sweep(other, model, oocc, 5, 0, 1, 0.07)
+    g = _captured(lambda: smc.sweep(lat, model, again, 5, 0, 2, kT))
+    g.replay()
+    torch.cuda.synchronize()
+    smc.check()
+    assert torch.equal(again, plain)
