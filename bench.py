@@ -453,8 +453,8 @@ def profile_fcc(n: int, nsweeps: int, qsro: bool = False):
 
 
 def profile_qsro(n: int, nsweeps: int):
-    """qSRO sweeps on an N^3 box (the count-cache kernel k_bq_cache, then 128
-    mini-step launches of k_bq_ministep per sweep), for ncu captures."""
+    """qSRO sweeps on an N^3 box (the count cache, then 32 launches of
+    k_qsro_group per sweep), for ncu captures."""
     import torch
     from paper_2604_08250_gb300 import build as _b
     from paper_2604_08250_gb300 import smc
@@ -640,7 +640,9 @@ def run_extras(smc, torch, dev, pk):
                       "frac_of_measured_bf16_sustained": tfl / pk["bf16_tflops_sustained"],
                       "flop_per_evaluated_attempt": MLP_FLOP_PER_ATTEMPT,
                       "note": "attempts with equal species (dE = 0) are not evaluated; evaluated_fraction is the "
-                              "unlike first-shell bond fraction before and after the timed sweeps"}
+                              "unlike first-shell bond fraction before and after the timed sweeps; a call of this "
+                              "size evaluates every feature vector once and looks f up, so the TFLOP/s count "
+                              "evaluations that are replaced by look-ups"}
     e4 = torch.zeros(1, dtype=torch.float64, device=dev)
     ems = timed(lambda: smc.energy(lat4, mlp_model, occ4, e4), reps=3)
     out["mlp_energy_256"] = {"ms": ems, "achieved_tflops": lat4.nsites * MLP_FLOP_PER_SITE_FWD / (ems * 1e-3) / 1e12}
@@ -676,9 +678,9 @@ def run_extras(smc, torch, dev, pk):
     zq = QSRO_ZONE[QSRO_SHELLS]
     bq = 2 + 2 * zq + accq * (2 + 2 + zq)
     out["qsro_256"] = {"cells": [256] * 3, "shells": QSRO_SHELLS, "sweeps_per_launch": nswq,
-                       "launches_per_sweep": 128, "ms_per_sweep": msq / nswq, "attempts_per_s": attq,
+                       "launches_per_sweep": 32, "ms_per_sweep": msq / nswq, "attempts_per_s": attq,
                        "accept_rate": accq, "bytes_per_attempt": bq, "achieved_gbs": attq * bq / 1e9,
-                       "note": "67 MB of species and count cache: L2-resident, bound by load latency"}
+                       "note": "rows of species and counts in shared memory for a group of four mini-steps: bound by issue"}
     eq = torch.zeros(1, dtype=torch.float64, device=dev)
     emsq = timed(lambda: smc.energy(latq, qm, occq, eq), reps=3)
     out["qsro_energy_256"] = {"ms": emsq}
@@ -690,7 +692,7 @@ def run_extras(smc, torch, dev, pk):
     msf = timed(lambda: smc.fcc_sweep(latf, fm, occf, 1, 0, nswf, kTf, n_acc=nf), reps=1)
     Nf = smc.fcc_nsites(latf)
     out["fcc_256"] = {"cells": [256] * 3, "sites": Nf, "shells": 2, "sweeps_per_launch": nswf,
-                      "launches_per_sweep": 256, "ms_per_sweep": msf / nswf,
+                      "launches_per_sweep": 64, "ms_per_sweep": msf / nswf,
                       "attempts_per_s": Nf * nswf / (msf * 1e-3),
                       "accept_rate": float(nf.item()) / (2 * Nf * nswf)}
     ef = torch.zeros(1, dtype=torch.float64, device=dev)
@@ -703,7 +705,7 @@ def run_extras(smc, torch, dev, pk):
     msq = timed(lambda: smc.fcc_sweep(latq, qm, occq, 1, 0, nswq, kTq, n_acc=nq), reps=1)
     Nq = smc.fcc_nsites(latq)
     out["fcc_qsro_256"] = {"cells": [256] * 3, "sites": Nq, "shells": 2, "composition": "Fe29Co29Ni28Al7Ti7",
-                           "sweeps_per_launch": nswq, "launches_per_sweep": 256, "ms_per_sweep": msq / nswq,
+                           "sweeps_per_launch": nswq, "launches_per_sweep": 64, "ms_per_sweep": msq / nswq,
                            "attempts_per_s": Nq * nswq / (msq * 1e-3),
                            "accept_rate": float(nq.item()) / (2 * Nq * nswq),
                            "paper_context_attempts_per_s": {"H100 SMC-X": 3.71e7, "H100 SMC-AI": 1.87e7}}
