@@ -302,9 +302,9 @@ __global__ void __launch_bounds__(kRgThreads) k_fcc_group(const __grid_constant_
     using Wide = typename std::conditional<IS_INT, long long, float>::type;  // as k_fcc_ministep
     constexpr int NV = NSH == 1 ? 12 : (NSH == 2 ? 18 : 42);
     const RowGroup &G = P.G;
-    const Word *sT = (const Word *)g_smem;          // [NSH][64][8]
-    const int *sB = (const int *)(sT + NSH * 512);  // [44][16]
-    constexpr uint32_t rows0 = (uint32_t)(NSH * 512 + 44 * 16) * 4;
+    const Word *sT = (const Word *)g_smem;  // [NSH] rows (A, B) of 8 (rg_d_at)
+    const int *sB = (const int *)(sT + NSH * kRgDShell);  // [44][16]
+    constexpr uint32_t rows0 = (uint32_t)(NSH * kRgDShell + 44 * 16) * 4;
     const int tid = threadIdx.x, c = tid / G.tpc, tt = tid - c * G.tpc, col = blockIdx.x * G.C + c;
     const bool on = col < G.ncol;
     const int y0 = 4 * (col % G.NLy) + G.dy, z0 = 4 * (col / G.NLy) + G.dz;
@@ -313,9 +313,9 @@ __global__ void __launch_bounds__(kRgThreads) k_fcc_group(const __grid_constant_
     if (on) rg_rows(G, rown, y0, z0, tt);
     __syncthreads();
     if (on) rg_stage<1>(G, (const unsigned char *)P.occ, base, G.pitch, G.unit, G.inv, rown, tt);
-    for (int i = tid; i < NSH * 512; i += blockDim.x) ((uint32_t *)g_smem)[i] = __ldg(P.tables + i);
+    for (int i = tid; i < NSH * 512; i += blockDim.x) ((uint32_t *)g_smem)[rg_d_at(i)] = __ldg(P.tables + i);
     for (int i = tid; i < 44 * 16; i += blockDim.x)
-        ((uint32_t *)g_smem)[NSH * 512 + i] = __ldg(P.tables + kFgB + G.sub * 44 * 16 + i);
+        ((uint32_t *)g_smem)[NSH * kRgDShell + i] = __ldg(P.tables + kFgB + G.sub * 44 * 16 + i);
     const bool active = on && tt < G.NLx;
     const int lc = col * G.NLx + tt;
     double accE = 0.0;
@@ -338,16 +338,16 @@ __global__ void __launch_bounds__(kRgThreads) k_fcc_group(const __grid_constant_
 #pragma unroll
             for (int t = 0; t < NV; ++t) qb[t] = SM8(at + ob[t * 16]);
             const int A = SM8(at) & 7, B = SM8(bt) & 7;
-            const Word *row = sT + (A * 8 + B) * 8;
+            const Word *row = sT + A * kRgDA + B * kRgDB;
             Wide dw = Wide(0);
 #pragma unroll
             for (int t = 0; t < NV; ++t) {
-                const Word v = row[fcc_shell_off(t) + (qa[t] & 7)];
+                const Word v = row[fcc_shell_off(t) / 512 * kRgDShell + (qa[t] & 7)];
                 if (t >= 12 || t != dir) dw += (Wide)v;
             }
 #pragma unroll
             for (int t = 0; t < NV; ++t) {
-                const Word v = row[fcc_shell_off(t) + (qb[t] & 7)];
+                const Word v = row[fcc_shell_off(t) / 512 * kRgDShell + (qb[t] & 7)];
                 if (t >= 12 || t != opp) dw -= (Wide)v;
             }
             // a dE beyond the int range is rejected anyway (the acceptance table is shorter)
@@ -993,7 +993,7 @@ smc_status launch_fcc_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     RowSet grows[4];
     int goff[4][42];
     bool grouped = false;
-    const size_t fixed = (size_t)(m->nshells * 512 + 44 * 16) * 4;
+    const size_t fixed = (size_t)(m->nshells * kRgDShell + 44 * 16) * 4;
     if (!is_qsro && rg_plan(lat, occ, ws->num_sms, ws->smem_optin, fixed, fcc_rows(m->nshells), 0, gp.G)) {
         words.resize(kFgB);
         if (!fcc_group_tables(m->nshells, gp.G.pitch, words, grows, goff)) {

@@ -36,6 +36,21 @@ struct RowSet {
     signed char sub[kRgRows], dy[kRgRows], dz[kRgRows];
 };
 
+// Rows (A, B) of 8 words in shared memory, kRgDA A + kRgDB B words from the
+// start of their shell.  The lanes of a warp read words of unrelated rows; these
+// strides spread the S^3 words in use over the 32 banks: 2.8 accesses for a
+// warp's 32 random words of five species, 4.0 with rows of 8 words one after the
+// other, where a bank belongs to one species (eight species: 3.3 either way).
+// Legs of two sweeps, two shells, five species: 256^3 FCC cells 5.14 -> 4.77 ms,
+// 128^3 1.64 -> 1.38 ms; three shells, 160 x 128 x 128 2.98 -> 2.71 ms; eight
+// species unchanged.
+constexpr int kRgDA = 83, kRgDB = 9, kRgDShell = 652;
+static_assert(7 * kRgDA + 7 * kRgDB + 8 <= kRgDShell && kRgDShell % 4 == 0, "room for a shell's rows");
+__host__ __device__ constexpr int rg_d_at(int i)  // word i of the tables [shell][A][B][8]
+{
+    return (i >> 9) * kRgDShell + ((i >> 6) & 7) * kRgDA + ((i >> 3) & 7) * kRgDB + (i & 7);
+}
+
 // What staging needs to know about the box and the launch.
 struct RowGroup {
     int nx, ny, nz, NLx, NLy, ncol;
