@@ -93,7 +93,7 @@ __device__ __forceinline__ int32_t cta_band(float cx)
 
 template <bool IS_INT, int NSH, int LPT>
 __device__ void cta_compute(const SweepParams &P, const CtaLayout &L, const RepDesc &RD, int tid, long long &accE,
-                            int &accN, int rep)
+                            long long &accN, int rep)
 {
     constexpr int NV = NSH >= 3 ? 26 : 14;
     constexpr int kTerms = (2 * NV + LPT - 1) / LPT;
@@ -120,6 +120,7 @@ __device__ void cta_compute(const SweepParams &P, const CtaLayout &L, const RepD
     }
     int half = 0;
     for (int t = 0; t < P.nsweeps; ++t) {
+        int accS = 0;  // accepted trials of this sweep (at most the lattice's sites; a launch's exceed 32 bits)
         float cx = 0.f;
         int32_t band = 0;  // floating-point models: dE in (lo, lo + band] needs the exact test
         if constexpr (!IS_INT) {
@@ -197,7 +198,7 @@ __device__ void cta_compute(const SweepParams &P, const CtaLayout &L, const RepD
                     }
                     if (lane == 0) {
                         accE += s;
-                        ++accN;
+                        ++accS;
                     }
                 }
                 if (one_warp)
@@ -206,6 +207,7 @@ __device__ void cta_compute(const SweepParams &P, const CtaLayout &L, const RepD
                     asm volatile("bar.sync 1, %0;" ::"r"(L.cthr) : "memory");
             }
         }
+        accN += accS;
     }
 }
 
@@ -317,8 +319,7 @@ __global__ void k_sweep_cta(const __grid_constant__ SweepParams P, int check)
         occ[i] = (unsigned char)(v & 7);
     }
     if (bad && check) atomicCAS(P.status, 0, (int)SMC_ERR_ARG);
-    long long accE = 0;
-    int accN = 0;
+    long long accE = 0, accN = 0;
     if (tid >= L.cthr) {
         // (threads of a larger replica's block that this one does not need draw words as well)
         __syncthreads();  // the compute warps read the offset table
