@@ -64,7 +64,11 @@
  * stream is synchronised.  The library owns a per-device workspace (link-cell
  * progress flags, partial sums, acceptance tables) that it grows with
  * cudaMalloc when needed and never frees before process exit; calls that use
- * it must not run concurrently on different streams of one device.
+ * it must not run concurrently on different streams of one device.  A call
+ * captured into a CUDA graph must not have to grow it (make the call once
+ * before), and host tables and weights that it copies are read again at every
+ * replay.  The buffers that a captured call used stay allocated when a later
+ * call needs larger ones, so the graph stays valid.
  *
  * Errors.  Argument errors return synchronously and leave every buffer
  * untouched.  Device-side failures (a progress wait that exceeded its time

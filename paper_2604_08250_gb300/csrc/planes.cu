@@ -357,20 +357,24 @@ void *planes_buffer(int which, size_t bytes, cudaStream_t stream)
     static void *bufs[2];
     static size_t caps[2];
     static int devs[2] = {-1, -1};
+    static bool held[2];
     void *&buf = bufs[which];
     int d = 0;
     if (cudaGetDevice(&d) != cudaSuccess) return nullptr;
-    if (buf && bytes <= caps[which] && d == devs[which]) return buf;
-    if (stream_capturing(stream) || cudaDeviceSynchronize() != cudaSuccess) return nullptr;
-    void *p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+    if (!buf || bytes > caps[which] || d != devs[which]) {
+        if (stream_capturing(stream) || cudaDeviceSynchronize() != cudaSuccess) return nullptr;
+        void *p = nullptr;
+        if (cudaMalloc(&p, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        release(buf, held[which]);
+        buf = p;
+        caps[which] = bytes;
+        devs[which] = d;
+        held[which] = false;
     }
-    if (buf) cudaFree(buf);
-    buf = p;
-    caps[which] = bytes;
-    devs[which] = d;
+    if (call_captured()) held[which] = true;
     return buf;
 }
 

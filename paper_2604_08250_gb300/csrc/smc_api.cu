@@ -42,6 +42,17 @@ int debug_fast_stage() { return g_fast_stage; }
 int debug_resident() { return g_resident; }
 
 static Workspace g_ws[64];
+static bool g_captured = false;  // the call under way is captured into a graph (under g_lock)
+
+bool call_captured() { return g_captured; }
+
+// Frees what a later launch no longer needs, unless a graph may still use it:
+// a captured call's addresses are in its graph, which can be replayed at any
+// time, so what it was given stays allocated until the process exits.
+void release(void *p, bool held)
+{
+    if (p && !held) cudaFree(p);
+}
 
 Workspace *workspace(smc_status *st)
 {
@@ -61,20 +72,22 @@ Workspace *workspace(smc_status *st)
             return nullptr;
         }
         const size_t cap = 1 << 20;
-        void *buf = nullptr;
+        void *buf = nullptr, *status = nullptr;
         e = cudaMalloc(&buf, cap);
+        if (e == cudaSuccess) e = cudaMalloc(&status, 256);
         if (e != cudaSuccess) {
             *st = cuda_fail(e, "cudaMalloc(workspace)");
+            cudaFree(buf);
             return nullptr;
         }
-        e = cudaMemset(buf, 0, 256);
+        e = cudaMemset(status, 0, 256);
         if (e != cudaSuccess) {
             *st = cuda_fail(e, "cudaMemset(workspace)");
             return nullptr;
         }
         ws->buf = buf;
         ws->cap = cap;
-        ws->status = (int *)buf;
+        ws->status = (int *)status;
         ws->num_sms = sms;
         ws->smem_optin = (size_t)optin;
         ws->device = dev;
@@ -83,44 +96,33 @@ Workspace *workspace(smc_status *st)
     return ws;
 }
 
-// Scratch starts 256 bytes into the buffer (after the status word).  Growing
-// frees the old buffer only after the device has finished with it.
+// Growing frees the old buffer only after the device has finished with it, and
+// not at all once a captured call has used it.  (Capacities double, so the
+// buffers kept for graphs are smaller together than the current one.)
 void *workspace_scratch(Workspace *ws, size_t bytes, smc_status *st)
 {
-    const size_t need = bytes + 256;
-    if (need > ws->cap) {
+    if (bytes > ws->cap) {
         cudaError_t e = cudaDeviceSynchronize();
         if (e != cudaSuccess) {
             *st = cuda_fail(e, "cudaDeviceSynchronize(workspace growth)");
             return nullptr;
         }
-        int status = 0;
-        e = cudaMemcpy(&status, ws->status, sizeof status, cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) {
-            *st = cuda_fail(e, "cudaMemcpy(status)");
-            return nullptr;
-        }
         size_t cap = ws->cap;
-        while (cap < need) cap *= 2;
+        while (cap < bytes) cap *= 2;
         void *buf = nullptr;
         e = cudaMalloc(&buf, cap);
         if (e != cudaSuccess) {
             *st = cuda_fail(e, "cudaMalloc(workspace)");
             return nullptr;
         }
-        e = cudaMemset(buf, 0, 256);
-        if (e == cudaSuccess) e = cudaMemcpy(buf, &status, sizeof status, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) {
-            *st = cuda_fail(e, "cudaMemset(workspace)");
-            return nullptr;
-        }
-        cudaFree(ws->buf);
+        release(ws->buf, ws->held);
         ws->buf = buf;
         ws->cap = cap;
-        ws->status = (int *)buf;
+        ws->held = false;
     }
+    if (g_captured) ws->held = true;
     *st = SMC_OK;
-    return (unsigned char *)ws->buf + 256;
+    return ws->buf;
 }
 
 bool lattice_valid(const smc_lattice *lat, bool mlp)
@@ -251,6 +253,10 @@ bool model_valid(const smc_lattice *lat, const smc_model *m)
 using namespace smc;
 
 #define API_LOCK std::lock_guard<std::mutex> _guard(g_lock)
+// Entry of a call that enqueues work on `stream`.
+#define API_ENTER(stream) \
+    API_LOCK;             \
+    g_captured = stream_capturing(stream)
 
 extern "C" {
 
@@ -352,7 +358,7 @@ smc_status smc_debug_set(int32_t what, int64_t value)
 smc_status smc_init_lattice(const smc_lattice *lat, const int64_t *counts, uint64_t seed, uint32_t replica,
                             int8_t *occ, cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     if (!lattice_valid(lat, false)) return SMC_ERR_ARG;
     if (!counts || !occ) {
         set_error("counts and occ must be non-NULL");
@@ -417,7 +423,7 @@ smc_status smc_sweep(const smc_lattice *lat, const smc_model *model, int8_t *occ
                      uint64_t sweep0, int32_t nsweeps, const double *kT, double *e_acc, int64_t *n_acc,
                      cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     smc_status st = check_sweep_args(lat, model, occ, nsweeps, kT, nsweeps, sweep0);
     if (st != SMC_OK) return st;
     if (nsweeps == 0) return SMC_OK;
@@ -470,7 +476,7 @@ smc_status smc_sweep_batched(int32_t R, const smc_lattice *lats, const smc_model
                              uint64_t seed, uint32_t replica0, uint64_t sweep0, int32_t nsweeps, const double *kT,
                              double *e_acc, int64_t *n_acc, cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     if (R < 1 || R > kMaxReplicas || !lats || !occ) {
         set_error("R must be in [1, %d] with lats and occ non-NULL", kMaxReplicas);
         return SMC_ERR_ARG;
@@ -501,7 +507,7 @@ smc_status smc_ministep_trace(const smc_lattice *lat, const smc_model *model, in
                               uint32_t replica, uint64_t sweep, int32_t k, double kT, float *dE, uint8_t *acc,
                               cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     smc_status st = check_sweep_args(lat, model, occ, 1, &kT, 1, sweep);
     if (st != SMC_OK) return st;
     const int nA = 2 * lc_edge(lat->nx) * lc_edge(lat->ny) * lc_edge(lat->nz);
@@ -520,7 +526,7 @@ smc_status smc_slab_ministep(const smc_lattice *lat, const smc_model *model, int
                              int32_t g, uint64_t seed, uint32_t replica, uint64_t sweep, int32_t k, double kT,
                              double *e_acc, int64_t *n_acc, int32_t part, cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     smc_status st = check_sweep_args(lat, model, win, 1, &kT, 1, sweep);
     if (st != SMC_OK) return st;
     if (model->kind != SMC_PAIR_I32 && model->kind != SMC_PAIR_F32) {
@@ -606,7 +612,7 @@ smc_status smc_fcc_sweep(const smc_lattice *lat, const smc_model *model, int8_t 
                          uint32_t replica, uint64_t sweep0, int32_t nsweeps, const double *kT, double *e_acc,
                          int64_t *n_acc, cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     smc_status st = fcc_check(lat, model, occ, true);
     if (st != SMC_OK) return st;
     if (nsweeps < 0 || nsweeps > (1 << 24)) {
@@ -641,7 +647,7 @@ smc_status smc_fcc_ministep_trace(const smc_lattice *lat, const smc_model *model
                                   uint32_t replica, uint64_t sweep, int32_t k, double kT, float *dE, uint8_t *acc,
                                   cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     smc_status st = fcc_check(lat, model, occ, true);
     if (st != SMC_OK) return st;
     if (k < 0 || k >= 256) {
@@ -666,7 +672,7 @@ smc_status smc_fcc_ministep_trace(const smc_lattice *lat, const smc_model *model
 smc_status smc_fcc_energy(const smc_lattice *lat, const smc_model *model, const int8_t *occ, double *e,
                           int64_t *e_int, cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     smc_status st = fcc_check(lat, model, occ, false);
     if (st != SMC_OK) return st;
     if (e_int && model->kind != SMC_PAIR_I32) {
@@ -679,7 +685,7 @@ smc_status smc_fcc_energy(const smc_lattice *lat, const smc_model *model, const 
 smc_status smc_sro(const smc_lattice *lat, int32_t nshells, const int8_t *occ, int64_t *counts, double *alpha,
                    cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     if (!lattice_valid(lat, false)) return SMC_ERR_ARG;
     if (nshells < 1 || nshells > kMaxShells || !occ) {
         set_error("nshells must be in [1, 3] and occ non-NULL");
@@ -701,7 +707,7 @@ smc_status smc_sro(const smc_lattice *lat, int32_t nshells, const int8_t *occ, i
 smc_status smc_energy(const smc_lattice *lat, const smc_model *model, const int8_t *occ, double *e, int64_t *e_int,
                       cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     if (!lattice_valid(lat, model && is_mlp(model)) || !model_valid(lat, model)) return SMC_ERR_ARG;
     if (!occ) {
         set_error("occ is NULL");
@@ -745,7 +751,7 @@ int64_t smc_grad_size(const smc_lattice *lat, const smc_model *model)
 smc_status smc_energy_grad(const smc_lattice *lat, const smc_model *model, const int8_t *occ, float *grad,
                            cudaStream_t stream)
 {
-    API_LOCK;
+    API_ENTER(stream);
     if (!lattice_valid(lat, model && is_mlp(model)) || !model_valid(lat, model)) return SMC_ERR_ARG;
     if (!occ || !grad) {
         set_error("occ and grad must be non-NULL");

@@ -147,13 +147,18 @@ struct Workspace {
     int device = -1;
     void *buf = nullptr;
     size_t cap = 0;
-    int *status = nullptr;  // latched device status (first 16 bytes of buf)
+    bool held = false;      // a graph may hold buf
+    int *status = nullptr;  // latched device status (never moves)
     int num_sms = 0;
     size_t smem_optin = 0;
 };
 Workspace *workspace(smc_status *st);
-// Ensures at least `bytes` of scratch after the status header; returns it.
+// Ensures at least `bytes` of scratch; returns it.
 void *workspace_scratch(Workspace *ws, size_t bytes, smc_status *st);
+// Whether the call under way is captured into a graph; frees a device buffer
+// unless a captured call was given it (held).
+bool call_captured();
+void release(void *p, bool held);
 // Whether the stream is being captured into a graph (or cannot tell).
 inline bool stream_capturing(cudaStream_t stream)
 {

@@ -423,7 +423,6 @@ smc_status launch_pair_sweep_cta(int R, const smc_lattice *lats, const smc_model
         e = cudaMemcpyAsync(scr, tabs.data(), tabs.size() * 4, cudaMemcpyHostToDevice, stream);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(acceptance tables)");
         P.tab = (const uint32_t *)scr;
-        P.status = ws->status;  // (the workspace may have moved)
     }
     auto kern = is_int ? (pt.nsh >= 3 ? k_sweep_cta<true, 3> : k_sweep_cta<true, 2>)
                        : (pt.nsh >= 3 ? k_sweep_cta<false, 3> : k_sweep_cta<false, 2>);

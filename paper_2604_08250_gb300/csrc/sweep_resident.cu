@@ -1007,6 +1007,7 @@ struct ResWave {
 
 struct ResMulti {
     bool ok = false;
+    bool held = false;     // a graph may hold the waves' lists
     int ncols = kResCols;  // compute warps per CTA
     const void *kernel = nullptr;
     std::vector<ResPlan> rp;
@@ -1015,9 +1016,9 @@ struct ResMulti {
 
 void free_waves(ResMulti &mp)
 {
-    for (auto &w : mp.waves)
-        if (w.dev) cudaFree(w.dev);
+    for (auto &w : mp.waves) release(w.dev, mp.held);
     mp.waves.clear();
+    mp.held = false;
 }
 
 // Compute warps per CTA for R replicas.  A wave's time is its groups', 2.77 us
@@ -1236,6 +1237,7 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
     }
     const ResMulti &mp = plan_cached;
     if (!mp.ok) return SMC_ERR_UNSUPPORTED;
+    if (call_captured()) plan_cached.held = true;
 
     // per-sweep temperatures: one launch per kMaxBeta / (replicas of the wave) sweeps
     bool constant = true;
