@@ -660,16 +660,22 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
         set_error("internal error: MLP interaction-zone geometry");
         return SMC_ERR_STATE;
     }
-    // workspace: [part_e | part_n | abort | weights | moves | ranks | packed counts | feature words | zone | D | state | table]
+    // workspace: [part_e | part_n | abort | weights | moves | ranks | packed counts | feature words | zone | D | state];
+    // the table (4 bytes per vector, whatever the lattice) has a buffer of its own
     const size_t nc = (size_t)P.NLx * P.ncol, N = 2ull * lat->nx * lat->ny * lat->nz;
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t o_pn = nc * 8, o_abort = o_pn + nc * 8, o_w = up(o_abort + 16), o_mv = up(o_w + kWeightBytes),
                  o_rk = up(o_mv + T.moves.size() * 2), o_un = up(o_rk + T.ranks.size() * 2),
                  o_rows = up(o_un + T.unrank.size() * 4), o_zone = up(o_rows + T.rows.size() * 4), o_D = up(o_zone + zone.size() * 4),
-                 o_red = up(o_D + kDEntries * 4), o_state = up(o_red + lc_reduce_bytes()), o_tab = up(o_state + N * 8),
-                 need = std::max(o_tab + (size_t)T.d.entries * 4, least);
+                 o_red = up(o_D + kDEntries * 4), o_state = up(o_red + lc_reduce_bytes()),
+                 need = std::max(o_state + N * 8, least);
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, need, &st);
     if (!scr) {  // no room for the table: the evaluating sweep needs none
+        cudaGetLastError();
+        return SMC_OK;
+    }
+    void *table = nullptr;
+    if (table_buffer((size_t)T.d.entries * 4, &table) != cudaSuccess) {
         cudaGetLastError();
         return SMC_OK;
     }
@@ -678,7 +684,7 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
     P.part_n = (long long *)(scr + o_pn);
     P.occ = occ;
     P.state = (uint2 *)(scr + o_state);
-    P.table = (const float *)(scr + o_tab);
+    P.table = (const float *)table;
     P.moves = (const uint16_t *)(scr + o_mv);
     P.ranks = (const uint16_t *)(scr + o_rk);
     P.unrank = (const uint32_t *)(scr + o_un);
@@ -701,8 +707,8 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
     put(o_zone, zone.data(), zone.size() * 4);
     if (pair) put(o_D, D, kDEntries * 4);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(MLP table sweep)");
-    st = net ? fill_launch<NetRelu96>(ws, scr + o_w, T.d, (const uint4 *)(scr + o_rows), (float *)(scr + o_tab), (int *)(scr + o_abort), stream)
-             : fill_launch<NetSilu64>(ws, scr + o_w, T.d, (const uint4 *)(scr + o_rows), (float *)(scr + o_tab), (int *)(scr + o_abort), stream);
+    st = net ? fill_launch<NetRelu96>(ws, scr + o_w, T.d, (const uint4 *)(scr + o_rows), (float *)table, (int *)(scr + o_abort), stream)
+             : fill_launch<NetSilu64>(ws, scr + o_w, T.d, (const uint4 *)(scr + o_rows), (float *)table, (int *)(scr + o_abort), stream);
     if (st != SMC_OK) return st;
     const int sb = (int)std::max<size_t>(1, std::min<size_t>((N + 255) / 256, (size_t)ws->num_sms * 64));
     k_table_state<<<sb, 256, 0, stream>>>(P);

@@ -364,7 +364,7 @@ void *planes_buffer(int which, size_t bytes, cudaStream_t stream)
     if (!buf || bytes > caps[which] || d != devs[which]) {
         if (stream_capturing(stream) || cudaDeviceSynchronize() != cudaSuccess) return nullptr;
         void *p = nullptr;
-        if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        if (device_alloc(&p, bytes) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }

@@ -42,6 +42,12 @@ int debug_fast_stage() { return g_fast_stage; }
 int debug_resident() { return g_resident; }
 
 static Workspace g_ws[64];
+struct TableBuffer {
+    void *buf = nullptr;
+    size_t cap = 0;
+};
+static TableBuffer g_table[64];           // by device
+static cudaError_t g_alloc_error = cudaSuccess;  // what the next allocation is made to return (debug)
 static bool g_captured = false;  // the call under way is captured into a graph (under g_lock)
 
 bool call_captured() { return g_captured; }
@@ -52,6 +58,52 @@ bool call_captured() { return g_captured; }
 void release(void *p, bool held)
 {
     if (p && !held) cudaFree(p);
+}
+
+static cudaError_t table_free(int dev)
+{
+    cudaError_t e = cudaDeviceSynchronize();  // kernels of an earlier call may read it
+    if (e == cudaSuccess) e = cudaFree(g_table[dev].buf);
+    if (e == cudaSuccess) g_table[dev] = TableBuffer();
+    return e;
+}
+
+static cudaError_t try_malloc(void **p, size_t bytes)
+{
+    const cudaError_t injected = g_alloc_error;
+    g_alloc_error = cudaSuccess;
+    return injected != cudaSuccess ? injected : cudaMalloc(p, bytes);
+}
+
+cudaError_t device_alloc(void **p, size_t bytes)
+{
+    cudaError_t e = try_malloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();  // (not sticky)
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64 || !g_table[dev].buf) return e;
+    const cudaError_t freed = table_free(dev);
+    if (freed != cudaSuccess) return freed;
+    e = try_malloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
+}
+
+cudaError_t table_buffer(size_t bytes, void **p)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && dev >= 64) e = cudaErrorInvalidDevice;
+    if (e != cudaSuccess) return e;
+    TableBuffer &t = g_table[dev];
+    if (bytes > t.cap) {
+        if (t.buf) e = table_free(dev);
+        if (e == cudaSuccess) e = device_alloc(&t.buf, bytes);
+        if (e != cudaSuccess) return e;
+        t.cap = bytes;
+    }
+    *p = t.buf;
+    return cudaSuccess;
 }
 
 Workspace *workspace(smc_status *st)
@@ -73,8 +125,8 @@ Workspace *workspace(smc_status *st)
         }
         const size_t cap = 1 << 20;
         void *buf = nullptr, *status = nullptr;
-        e = cudaMalloc(&buf, cap);
-        if (e == cudaSuccess) e = cudaMalloc(&status, 256);
+        e = device_alloc(&buf, cap);
+        if (e == cudaSuccess) e = device_alloc(&status, 256);
         if (e != cudaSuccess) {
             *st = cuda_fail(e, "cudaMalloc(workspace)");
             cudaFree(buf);
@@ -110,7 +162,7 @@ void *workspace_scratch(Workspace *ws, size_t bytes, smc_status *st)
         size_t cap = ws->cap;
         while (cap < bytes) cap *= 2;
         void *buf = nullptr;
-        e = cudaMalloc(&buf, cap);
+        e = device_alloc(&buf, cap);
         if (e != cudaSuccess) {
             *st = cuda_fail(e, "cudaMalloc(workspace)");
             return nullptr;
@@ -349,6 +401,14 @@ smc_status smc_debug_set(int32_t what, int64_t value)
             return SMC_ERR_ARG;
         }
         g_resident = (int)value;
+        return SMC_OK;
+    }
+    if (what == SMC_DBG_ALLOC_ERROR) {
+        if (value < 0 || value > 999) {
+            set_error("allocation error must be a cudaError_t");
+            return SMC_ERR_ARG;
+        }
+        g_alloc_error = (cudaError_t)value;
         return SMC_OK;
     }
     set_error("unknown debug key %d", what);

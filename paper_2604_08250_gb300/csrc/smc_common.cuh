@@ -159,6 +159,12 @@ void *workspace_scratch(Workspace *ws, size_t bytes, smc_status *st);
 // unless a captured call was given it (held).
 bool call_captured();
 void release(void *p, bool held);
+// cudaMalloc for every buffer that the library keeps.  Without room the table
+// buffer is given back first.
+cudaError_t device_alloc(void **p, size_t bytes);
+// The buffer of the tabulated MLP sweeps (exactly the size of the largest
+// table so far, apart from the workspace, never in a graph).
+cudaError_t table_buffer(size_t bytes, void **p);
 // Whether the stream is being captured into a graph (or cannot tell).
 inline bool stream_capturing(cudaStream_t stream)
 {

@@ -1169,7 +1169,7 @@ smc_status build_res_multi(int R, const smc_lattice *lats, const PairTable &pt, 
             w.ver_words += (size_t)2 * rp.nver * (size_t)(((l.nx + 7) / 8) * 2);
         }
         w.lists_off = (desc.size() * 4 + 15) / 16 * 16;
-        e = cudaMalloc(&w.dev, w.lists_off + lists.size() * 4);
+        e = device_alloc(&w.dev, w.lists_off + lists.size() * 4);
         if (e == cudaSuccess) e = cudaMemcpy(w.dev, desc.data(), desc.size() * 4, cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
             e = cudaMemcpy((unsigned char *)w.dev + w.lists_off, lists.data(), lists.size() * 4,
