@@ -697,8 +697,11 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
     st = mlp_copy_weights(m, scr + o_w, stream);
     if (st != SMC_OK) return st;
     cudaError_t e = cudaMemsetAsync(scr, 0, o_abort + 16, stream);
+    // (in pieces: a copy of more than 64 KB of pageable memory waits for the work ahead of it on the stream)
     auto put = [&](size_t off, const void *src, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMemcpyAsync(scr + off, src, bytes, cudaMemcpyHostToDevice, stream);
+        for (size_t o = 0; o < bytes && e == cudaSuccess; o += 32768)
+            e = cudaMemcpyAsync(scr + off + o, (const char *)src + o, std::min<size_t>(32768, bytes - o),
+                                cudaMemcpyHostToDevice, stream);
     };
     put(o_mv, T.moves.data(), T.moves.size() * 2);
     put(o_rk, T.ranks.data(), T.ranks.size() * 2);
