@@ -166,14 +166,16 @@ smc_status smc_init_lattice(const smc_lattice *lat, const int64_t *counts, uint6
  * interaction zone of every accepted swap, so a trial evaluates only the 40
  * post-swap energies of its zone, and the per-site features (species and
  * per-shell species counts, 16 N bytes) the same way; they need every axis
- * a multiple of 4 cells and >= 8, nx <= 1024.  A call that would evaluate
- * more rows than there are feature vectors (9.5e8 for five species: about
- * one sweep of 256^3; MLPNet half as many) evaluates every vector once and
- * looks the others up (8 N bytes of workspace and 4 bytes per vector in a
- * buffer of its own, 3.8 GB for five species, which is kept for later calls and
- * given back when another allocation of the library finds no room; without
- * room for it, and into a CUDA graph, it runs as a smaller call does), with
- * the same results bit for bit.  qSRO models keep each site's own-species
+ * a multiple of 4 cells and >= 8, nx <= 1024.  A call of enough
+ * sweeps of a lattice with enough unlike neighbours (five species in equal
+ * parts: from about one sweep of 256^3 on, and never below about 32^3; counted
+ * on the device when the call starts, without waiting for it) evaluates f for
+ * every feature vector once (9.5e8 for five species) and looks it up (8 N
+ * bytes of workspace and 4 bytes per vector in a buffer of its own, 3.8 GB for
+ * five species, which is kept for later calls and given back when another
+ * allocation of the library finds no room; without room for it, and into a
+ * CUDA graph, it evaluates as a smaller call does), with the same results bit
+ * for bit.  qSRO models keep each site's own-species
  * count per shell (N bytes for 1-2 shells, 2 N for 3), built at the start of
  * every call and updated by accepted swaps (boxes of up to 1024 cells per row
  * run the four mini-steps of a group in one launch); a trial's dE comes
@@ -384,8 +386,9 @@ smc_status smc_set_tuning(const smc_tuning *t);
  * cells on every axis (0 = automatic); SMC_DBG_RESIDENT = 1 keeps the pair
  * sweep from holding a small lattice in shared memory for a whole call
  * (0 = automatic); SMC_DBG_ALLOC_ERROR makes the library's next device
- * allocation return that cudaError_t without being tried (0 = off).  Results
- * never depend on them. */
+ * allocation return that cudaError_t without being tried (0 = off);
+ * SMC_DBG_MLP_TABLE fixes the route of MLP sweeps (1: evaluating, 2: tabulated
+ * where the table fits, 0 = automatic).  Results never depend on them. */
 enum {
     SMC_DBG_TIMEOUT_MS = 1,
     SMC_DBG_SKIP_PUBLISH = 2,
@@ -393,7 +396,8 @@ enum {
     SMC_DBG_FAST_BUFFERS = 4,
     SMC_DBG_FAST_STAGING = 5,
     SMC_DBG_RESIDENT = 6,
-    SMC_DBG_ALLOC_ERROR = 7
+    SMC_DBG_ALLOC_ERROR = 7,
+    SMC_DBG_MLP_TABLE = 8
 };
 smc_status smc_debug_set(int32_t what, int64_t value);
 

@@ -12,7 +12,8 @@
 // evaluated (mlp_tc.cuh), so the looked-up sweep takes the same decisions as
 // the evaluating one.  Measured (GB300, 256^3, five species): the table 35 ms
 // (MLP) or 36 ms (MLPNet), then 22 ms per sweep, against 60 ms (MLP) and 90 ms
-// (MLPNet) per sweep of the evaluating kernel.
+// (MLPNet) per sweep of the evaluating kernel.  Which of the two a call takes
+// depends on the box and on its share of unlike bonds (table_gain).
 //
 // Feature vectors are numbered shell by shell: r_m is the rank of the shell's
 // composition among the n_m, most probable (largest multinomial coefficient)
@@ -189,6 +190,7 @@ struct TableParams {
     uint32_t replica;
     float beta;
     int g;                   // group
+    const int *route;        // 0 there: the call evaluates its rows, nothing to do here (NULL: tabulated for certain)
     int *status;
     long long timeout_ns;
 };
@@ -238,8 +240,10 @@ __device__ __forceinline__ uint32_t word_index(const TableDims &D, uint32_t w)
 template <class Net>
 __global__ void __launch_bounds__(128 * Net::kFillNWG) k_table_fill(const void *W, const TableDims D,
                                                               const uint4 *__restrict__ rows, float *table,
-                                                              long long timeout_ns, int *status, int *abort_flag)
+                                                              const int *route, long long timeout_ns, int *status,
+                                                              int *abort_flag)
 {
+    if (route && *route == 0) return;
     constexpr int NWG = Net::kFillNWG;
     constexpr uint32_t xg = NWG <= 4 ? 512 : 384;  // bytes of 8 rows of the X tile
     typename Net::Eval E = mlp_evaluator<Net, NWG>(timeout_ns, status, abort_flag);
@@ -311,6 +315,7 @@ __device__ __forceinline__ int state_pos(int x, int NLx) { return (x & 3) * NLx 
 // The state of every site from the occupancy.
 __global__ void __launch_bounds__(256) k_table_state(const __grid_constant__ TableParams P)
 {
+    if (P.route && *P.route == 0) return;
     const long long N = 2LL * P.nx * P.ny * P.nz;
     const int S = P.d.S;
     auto spec = [&](int sb, int xx, int yy, int zz) { return occ_at(P.occ, P.nx, P.ny, P.nz, sb, xx, yy, zz); };
@@ -409,6 +414,7 @@ __device__ __forceinline__ void team_sync(int team, int n)
 template <bool HAS_PAIR, bool SPLIT>
 __global__ void __launch_bounds__(kTabThreads, 1) k_table_sweep(const __grid_constant__ TableParams P)
 {
+    if (P.route && *P.route == 0) return;
     // shared memory: moves | zone table | the moves' offsets | progress | (pair) D | per team: row numbers,
     // Philox words, rows
     uint16_t *mv = (uint16_t *)g_smem;
@@ -579,7 +585,7 @@ size_t table_sweep_fixed(const TableDims &d, bool pair)
 
 template <class Net>
 smc_status fill_launch(Workspace *ws, const void *W, const TableDims &d, const uint4 *rows, float *table,
-                       int *abort_flag, cudaStream_t stream)
+                       const int *route, int *abort_flag, cudaStream_t stream)
 {
     constexpr int NWG = Net::kFillNWG;
     const size_t smem = (Net::template Smem<NWG>::TINFO + 127) / 128 * 128;
@@ -588,7 +594,7 @@ smc_status fill_launch(Workspace *ws, const void *W, const TableDims &d, const u
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_table_fill)");
     const long long tiles = (d.entries + kTcRows - 1) / kTcRows;
     const int grid = (int)std::max(1LL, std::min<long long>(ws->num_sms, (tiles + NWG - 1) / NWG));
-    kern<<<grid, 128 * NWG, smem, stream>>>(W, d, rows, table, debug_timeout_ns(), ws->status, abort_flag);
+    kern<<<grid, 128 * NWG, smem, stream>>>(W, d, rows, table, route, debug_timeout_ns(), ws->status, abort_flag);
     e = cudaGetLastError();
     return e == cudaSuccess ? SMC_OK : cuda_fail(e, "k_table_fill");
 }
@@ -615,23 +621,110 @@ bool pack_zone(int nx, std::vector<uint32_t> &out)
     return true;
 }
 
-}  // namespace
+// ---------------------------------------------------------------------------
+// The choice between evaluating and tabulating.  Both times follow the share
+// f of unlike first-shell bonds, since only trials of unlike species evaluate or
+// look up: a column of n trials has f n of them per mini-step, and none with
+// probability (1 - f)^n.  In us, fitted to 23 boxes of 8^3 to 256^3 cells (cubes,
+// single columns and plates), two, four and five species, f = 0.02 to 0.8, to
+// 12 % (root mean square):
+//   evaluating  per mini-step of a column
+//               1.65 + 1.55 (1 - (1 - f)^n) + 0.28 f n (MLPNet: 0.46 f n) + 0.0085 n,
+//               columns one after the other on an SM;
+//   tabulated   per group of a block's K columns (c0..c3)
+//               c0 + c1 (1 - (1 - f)^n) + (c2 f + c3) K n,
+//               and per call 37 ps per vector (the table) and 60 us (launches, copies).
+// Over these boxes and calls of 1 to 5000 sweeps the slower route is taken, by
+// more than 5 %, for 1 in 100; with the rows of an alloy in equal parts over the
+// number of vectors alone it was 1 in 6.  Per call, evaluating / tabulated (ms):
+//   256^3, 2 sweeps: Dirichlet fractions 122 / 84, 1 % of one solute 26 / 49
+//   128^3, 12 sweeps: Dirichlet 102 / 78, two of five species 82 / 54, 1 % 26 / 49
+//   32^3, 600 sweeps: equal fractions 389 / 566, 1 % 198 / 380; MLPNet 541 / 565
+//   16^3, 10 sweeps of three species 5.1 / 5.4; 64^3 15.9 / 6.0
+// f moves during a call (order sets in, or phases separate); the share at its
+// start decides.
+// ---------------------------------------------------------------------------
+struct TableGain {  // of tabulating (us): g0 + g1 (1 - (1 - f)^n) + g2 f
+    double g0, g1, g2, n;
+    __host__ __device__ double at(double f) const { return g0 + g1 * (1.0 - pow(1.0 - f, n)) + g2 * f; }
+};
 
-bool mlp_table_wanted(const smc_lattice *lat, const smc_model *m, int nsweeps)
+TableGain table_gain(int S, bool net, int nsweeps, int NLx, int eval_passes, int table_passes, int K, double entries)
 {
-    const TableDims &d = table_host(lat->nspecies).d;
-    const double evals = 2.0 * lat->nx * lat->ny * lat->nz * nsweeps * kOmega * (1.0 - 1.0 / lat->nspecies);
-    // Per row: 58 ps evaluated in the sweep (MLP; MLPNet 102), 21-25 looked up, 37 for a vector of the table: equal
-    // at 1.0-1.1 (0.45-0.5) times the vectors. MLPNet, 128^3:
-    // 3 sweeps evaluated 40.3 ms (looked up 47), 4 looked up 50.7 (evaluated 53.3), 7 looked up 61.5 (92.9).
-    return lat->nspecies >= 2 && evals > (m->kind == SMC_MLPNET_BF16 ? 0.55 : 1.15) * (double)d.entries;
+    static const double c[3][4] = {{10.6, 5.6, 0.05, 0.015}, {12.2, 5.5, 0.09, 0.0}, {14.7, 6.8, 0.26, 0.0}};
+    const double *t = c[S <= 3 ? 0 : S - 3];
+    const double ev = 128.0 * nsweeps * eval_passes, look = 32.0 * nsweeps * table_passes, kn = (double)K * NLx;
+    return TableGain{ev * (1.65 + 0.0085 * NLx) - look * (t[0] + t[3] * kn) - 37e-6 * entries - 60.0,
+                     ev * 1.55 - look * t[1], ev * (net ? 0.46 : 0.28) * NLx - look * t[2] * kn, (double)NLx};
 }
+
+// Unlike first-shell bonds, each once: sublattice 0's sites with their eight
+// neighbours, four cells of a row (a word) at a time (512^3: 0.19 ms, 0.71 by bytes).
+template <bool ALIGNED>
+__device__ __forceinline__ uint32_t four_species(const int8_t *p)
+{
+    if (ALIGNED) return *(const uint32_t *)p & 0x07070707u;
+    return (uint32_t)(p[0] & 7) | (uint32_t)(p[1] & 7) << 8 | (uint32_t)(p[2] & 7) << 16 | (uint32_t)(p[3] & 7) << 24;
+}
+
+template <bool ALIGNED>
+__global__ void __launch_bounds__(256) k_unlike_bonds(const int8_t *__restrict__ occ, int nx, int ny, int nz,
+                                                      unsigned long long *count)
+{
+    const uint32_t nw = (uint32_t)nx / 4, words = nw * ny * nz;  // rows are multiples of four cells; < 2^28
+    const int8_t *other = occ + 4 * (size_t)words;
+    uint32_t n = 0;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < words; i += gridDim.x * blockDim.x) {
+        const int w = (int)(i % nw), t = (int)(i / nw), y = t % ny, z = t / ny;
+        const uint32_t a = four_species<ALIGNED>(occ + 4 * (size_t)i);
+        const int left = w ? 4 * w - 1 : nx - 1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int8_t *row = other + (size_t)(wrapc(z - (k >> 1), nz) * ny + wrapc(y - (k & 1), ny)) * nx;
+            const uint32_t b = four_species<ALIGNED>(row + 4 * w), c = b << 8 | (uint32_t)(row[left] & 7);  // x, x - 1
+            n += __popc(__vcmpne4(a, b)) + __popc(__vcmpne4(a, c));
+        }
+    }
+    n = __reduce_add_sync(0xffffffffu, n / 8);  // eight bits per unlike pair
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, (unsigned long long)n);
+}
+
+__global__ void k_table_route(TableGain gain, double bonds, const unsigned long long *unlike, int *route)
+{
+    *route = gain.at((double)*unlike / bonds) > 0.0 ? 1 : 0;
+}
+
+// The route word's copy on the host.  The host never waits for it: it looks
+// before it enqueues each sweep, and what was enqueued before the word came
+// ends at once where it is not needed.
+struct RouteEcho {
+    int *word = nullptr;  // pinned
+    cudaEvent_t event = nullptr;
+};
+RouteEcho *route_echo()
+{
+    static RouteEcho echo[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return nullptr;
+    RouteEcho &r = echo[dev];
+    if (!r.word && cudaHostAlloc((void **)&r.word, sizeof(int), cudaHostAllocDefault) != cudaSuccess) r.word = nullptr;
+    if (!r.event && cudaEventCreateWithFlags(&r.event, cudaEventDisableTiming) != cudaSuccess) r.event = nullptr;
+    if (r.word && r.event) return &r;
+    cudaGetLastError();
+    return nullptr;
+}
+
+}  // namespace
 
 smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, int8_t *occ, uint64_t seed,
                                   uint32_t replica, uint64_t sweep0, int nsweeps, const double *kT, double *e_acc,
-                                  int64_t *n_acc, const float *D, size_t least, bool *taken, cudaStream_t stream)
+                                  int64_t *n_acc, const float *D, size_t least, int eval_passes, MlpTaken *taken,
+                                  const int **route, cudaStream_t stream)
 {
-    *taken = false;
+    *taken = kMlpEvaluate;
+    *route = nullptr;
+    const int fixed_route = debug_mlp_table();  // 0: chosen here; 1: evaluating; 2: tabulated where it fits
+    if (lat->nspecies < 2 || fixed_route == 1) return SMC_OK;
     smc_status st;
     Workspace *ws = workspace(&st);
     if (!ws) return st;
@@ -654,6 +747,12 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
     P.K = (int)std::min<size_t>((ws->smem_optin - fixed) / per,
                                 std::min({kTabThreads / P.team_threads, 15, (P.ncol + ws->num_sms - 1) / ws->num_sms}));
     const size_t smem = fixed + per * (size_t)P.K;
+    const int blocks = std::min(P.ncol, ws->num_sms), per_pass = blocks * P.K;
+    const TableGain gain = table_gain(lat->nspecies, net, nsweeps, P.NLx, eval_passes,
+                                      (P.ncol + per_pass - 1) / per_pass, P.K, (double)T.d.entries);
+    // worth a look at the lattice if it would be for a random alloy in equal parts
+    if (fixed_route == 0 && !(gain.at(1.0 - 1.0 / lat->nspecies) > 0.0)) return SMC_OK;
+    const bool certain = fixed_route == 2 || (gain.g0 > 0.0 && gain.g1 >= 0.0 && gain.g2 >= 0.0);  // for any lattice
     P.nshells = pair ? m->nshells : 0;
     std::vector<uint32_t> zone;
     if (!pack_zone(P.nx, zone)) {
@@ -675,11 +774,12 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
         return SMC_OK;
     }
     void *table = nullptr;
-    if (table_buffer((size_t)T.d.entries * 4, &table) != cudaSuccess) {
+    const size_t table_bytes = up((size_t)T.d.entries * 4);  // then the count and the route word
+    if (table_buffer(table_bytes + 16, &table) != cudaSuccess) {
         cudaGetLastError();
         return SMC_OK;
     }
-    *taken = true;
+    *taken = certain ? kMlpTabulate : kMlpEither;
     P.part_e = (double *)scr;
     P.part_n = (long long *)(scr + o_pn);
     P.occ = occ;
@@ -694,9 +794,40 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
     P.replica = replica;
     P.status = ws->status;
     P.timeout_ns = debug_timeout_ns();
+    cudaError_t e = cudaSuccess;
+    RouteEcho *echo = nullptr;
+    if (!certain) {
+        unsigned long long *unlike = (unsigned long long *)((unsigned char *)table + table_bytes);
+        int *word = (int *)(unlike + 1);
+        e = cudaMemsetAsync(unlike, 0, 16, stream);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(unlike bonds)");
+        const int cb = (int)std::max<size_t>(1, std::min<size_t>((N / 8 + 255) / 256, (size_t)ws->num_sms * 8));
+        if ((uintptr_t)occ % 4 == 0)
+            k_unlike_bonds<true><<<cb, 256, 0, stream>>>(occ, P.nx, P.ny, P.nz, unlike);
+        else
+            k_unlike_bonds<false><<<cb, 256, 0, stream>>>(occ, P.nx, P.ny, P.nz, unlike);
+        k_table_route<<<1, 1, 0, stream>>>(gain, 4.0 * (double)N, unlike, word);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(e, "k_table_route");
+        P.route = *route = word;
+        echo = route_echo();
+        if (echo) {
+            e = cudaMemcpyAsync(echo->word, word, sizeof(int), cudaMemcpyDeviceToHost, stream);
+            if (e == cudaSuccess) e = cudaEventRecord(echo->event, stream);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(route)");
+        }
+    }
+    // looks whether the route is known by now; false: the rest of the tabulated sweep is not needed
+    auto go_on = [&]() {
+        if (*taken != kMlpEither || !echo) return true;
+        const cudaError_t q = cudaEventQuery(echo->event);
+        if (q == cudaErrorNotReady) cudaGetLastError();
+        if (q == cudaSuccess) *taken = *(volatile int *)echo->word ? kMlpTabulate : kMlpEvaluate;
+        return *taken != kMlpEvaluate;
+    };
     st = mlp_copy_weights(m, scr + o_w, stream);
     if (st != SMC_OK) return st;
-    cudaError_t e = cudaMemsetAsync(scr, 0, o_abort + 16, stream);
+    e = cudaMemsetAsync(scr, 0, o_abort + 16, stream);
     // (in pieces: a copy of more than 64 KB of pageable memory waits for the work ahead of it on the stream)
     auto put = [&](size_t off, const void *src, size_t bytes) {
         for (size_t o = 0; o < bytes && e == cudaSuccess; o += 32768)
@@ -710,8 +841,8 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
     put(o_zone, zone.data(), zone.size() * 4);
     if (pair) put(o_D, D, kDEntries * 4);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(MLP table sweep)");
-    st = net ? fill_launch<NetRelu96>(ws, scr + o_w, T.d, (const uint4 *)(scr + o_rows), (float *)table, (int *)(scr + o_abort), stream)
-             : fill_launch<NetSilu64>(ws, scr + o_w, T.d, (const uint4 *)(scr + o_rows), (float *)table, (int *)(scr + o_abort), stream);
+    st = net ? fill_launch<NetRelu96>(ws, scr + o_w, T.d, (const uint4 *)(scr + o_rows), (float *)table, P.route, (int *)(scr + o_abort), stream)
+             : fill_launch<NetSilu64>(ws, scr + o_w, T.d, (const uint4 *)(scr + o_rows), (float *)table, P.route, (int *)(scr + o_abort), stream);
     if (st != SMC_OK) return st;
     const int sb = (int)std::max<size_t>(1, std::min<size_t>((N + 255) / 256, (size_t)ws->num_sms * 64));
     k_table_state<<<sb, 256, 0, stream>>>(P);
@@ -721,8 +852,9 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
                            : (pair ? k_table_sweep<true, false> : k_table_sweep<false, false>);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_table_sweep)");
-    const int blocks = std::min(P.ncol, ws->num_sms), threads = P.team_threads * P.K;
+    const int threads = P.team_threads * P.K;
     for (int t = 0; t < nsweeps; ++t) {
+        if (!go_on()) return SMC_OK;
         P.sweep = sweep0 + (uint64_t)t;
         P.beta = (float)(1.0 / kT[t]);
         for (int g = 0; g < 32; ++g) {
@@ -732,7 +864,8 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "k_table_sweep");
     }
-    if (e_acc || n_acc)
+    if (!go_on()) return SMC_OK;
+    if (e_acc || n_acc)  // (sums of zeros where the sweep was not needed)
         return launch_lc_reduce(P.part_e, P.part_n, (long long)nc, scr + o_red, e_acc, (long long *)n_acc, stream);
     return SMC_OK;
 }

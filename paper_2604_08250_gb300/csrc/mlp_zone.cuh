@@ -184,15 +184,19 @@ __device__ void mlp_cta_setup(typename Net::Eval &E, const void *W, const float 
 // pair table D of a pair + MLP model.
 bool build_mlp_geo(MlpGeo &G);
 smc_status mlp_copy_weights(const smc_model *m, void *dst, cudaStream_t stream);
-// Sweeps with f tabulated over all feature vectors (mlp_table.cu): whether a
-// call is large enough for it, and the call; *taken is false when the table
-// does not fit (the caller runs the evaluating sweep).  D: pair table (host).
-bool mlp_table_wanted(const smc_lattice *lat, const smc_model *m, int nsweeps);
-// (The workspace grows to `least` bytes at least: those of the evaluating
-// sweep, which takes the captured calls that a plain one prepares.)
+// Sweeps with f tabulated over all feature vectors (mlp_table.cu), where that
+// is the faster route.  *taken: kMlpEvaluate, the caller runs the evaluating
+// sweep (also when the table finds no room); kMlpTabulate, the call is done;
+// kMlpEither, the device decides by the lattice: the tabulated sweep runs if
+// **route is not 0, and the caller enqueues the evaluating one to run if it is.
+// D: pair table (host).  eval_passes: columns that a CTA of the evaluating
+// sweep takes in turn.  The workspace grows to `least` bytes at least: those of
+// the evaluating sweep, which shares it.
+enum MlpTaken { kMlpEvaluate, kMlpTabulate, kMlpEither };
 smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, int8_t *occ, uint64_t seed,
                                   uint32_t replica, uint64_t sweep0, int nsweeps, const double *kT, double *e_acc,
-                                  int64_t *n_acc, const float *D, size_t least, bool *taken, cudaStream_t stream);
+                                  int64_t *n_acc, const float *D, size_t least, int eval_passes, MlpTaken *taken,
+                                  const int **route, cudaStream_t stream);
 constexpr size_t kWeightBytes = sizeof(MlpBlock) > sizeof(NetBlock) ? sizeof(MlpBlock) : sizeof(NetBlock);
 
 }  // namespace smc

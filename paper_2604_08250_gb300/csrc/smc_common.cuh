@@ -183,6 +183,7 @@ int64_t debug_skip_tile();
 int debug_fast_team();
 int debug_fast_nbuf();
 int debug_fast_stage();
+int debug_mlp_table();
 
 bool lattice_valid(const smc_lattice *lat, bool mlp);
 bool model_valid(const smc_lattice *lat, const smc_model *m);

@@ -64,6 +64,7 @@ struct SweepParams {
     int lag[kMaxGroups];  // group g may start once neighbours completed g+1-lag[g] groups
     int warp_bytes;       // fast kernel: shared-memory bytes per warp
     int nap_cap;          // fast kernel: longest sleep between progress polls (ns)
+    const int *route;     // MLP sweep: not 0 there, the call's energies are looked up, nothing to do (NULL: evaluates)
     int kind;             // model kind (SMC_PAIR_I32 .. SMC_PAIR_F32_MLP_BF16)
     const void *mlpw;     // network weights (device MlpBlock or NetBlock), MLP kinds only
     float *ecache;        // per-site MLP energy f(x_i) (device, N floats), MLP kinds only

@@ -40,9 +40,10 @@ namespace smc {
 template <class Net>
 __global__ void __launch_bounds__(128 * kStreamWG) k_mlp_site_energy(const void *W, const int8_t *__restrict__ occ,
                                                                    int nx, int ny, int nz, float *ecache,
-                                                                   uint4 *fcache, double *part, long long timeout_ns,
-                                                                   int *status, int *abort_flag)
+                                                                   uint4 *fcache, double *part, const int *route,
+                                                                   long long timeout_ns, int *status, int *abort_flag)
 {
+    if (route && *route) return;  // a sweep whose energies are looked up
     constexpr int NWG = kStreamWG;
     using M = typename Net::template Smem<NWG>;
     typename Net::Eval E = mlp_evaluator<Net, NWG>(timeout_ns, status, abort_flag);
@@ -326,6 +327,7 @@ template <class Net, int MODE>
 __global__ void __launch_bounds__(128 * Net::kSweepNWG, 1) k_sweep_mlp(const __grid_constant__ SweepParams P,
                                                                        const __grid_constant__ MlpGeo G)
 {
+    if (P.route && *P.route) return;
     constexpr int NWG = Net::kSweepNWG, kThreads = 128 * NWG;
     using M = typename Net::template Smem<NWG>;
     typename Net::Eval E = mlp_evaluator<Net, NWG>(P.timeout_ns, P.status, P.abort_flag);
@@ -802,8 +804,8 @@ smc_status mlp_copy_weights(const smc_model *m, void *dst, cudaStream_t stream)
 // abort_flag is a device word that starts at zero.
 template <class Net>
 static smc_status mlp_energy_launch(Workspace *ws, const smc_lattice *lat, const void *W, const int8_t *occ,
-                                    float *ecache, uint4 *fcache, double *part, int *abort_flag, double *e,
-                                    int accumulate, cudaStream_t stream)
+                                    float *ecache, uint4 *fcache, double *part, const int *route, int *abort_flag,
+                                    double *e, int accumulate, cudaStream_t stream)
 {
     const size_t smem = Net::template Smem<kStreamWG>::END;
     auto kern = k_mlp_site_energy<Net>;
@@ -812,7 +814,7 @@ static smc_status mlp_energy_launch(Workspace *ws, const smc_lattice *lat, const
     const long long N = 2LL * lat->nx * lat->ny * lat->nz;
     const long long tiles = (N + kTcRows - 1) / kTcRows;
     const int grid = (int)std::max(1LL, std::min<long long>(ws->num_sms, tiles));
-    kern<<<grid, 128 * kStreamWG, smem, stream>>>(W, occ, lat->nx, lat->ny, lat->nz, ecache, fcache, part,
+    kern<<<grid, 128 * kStreamWG, smem, stream>>>(W, occ, lat->nx, lat->ny, lat->nz, ecache, fcache, part, route,
                                                            debug_timeout_ns(), ws->status, abort_flag);
     err = cudaGetLastError();
     if (err != cudaSuccess) return cuda_fail(err, "k_mlp_site_energy");
@@ -852,9 +854,9 @@ smc_status launch_mlp_energy(const smc_lattice *lat, const smc_model *m, const i
     }
     if (is_mlpnet(m))
         return mlp_energy_launch<NetRelu96>(ws, lat, scr + off_w, occ, nullptr, nullptr, (double *)(scr + off_part),
-                                            (int *)(scr + off_abort), e, accumulate, stream);
+                                            nullptr, (int *)(scr + off_abort), e, accumulate, stream);
     return mlp_energy_launch<NetSilu64>(ws, lat, scr + off_w, occ, nullptr, nullptr, (double *)(scr + off_part),
-                                        (int *)(scr + off_abort), e, accumulate, stream);
+                                        nullptr, (int *)(scr + off_abort), e, accumulate, stream);
 }
 
 namespace {
@@ -975,14 +977,15 @@ smc_status launch_mlp_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     const size_t off_cache =
         round16(off_parts + sizeof(double) * kTcMaxCtasPerSm * (size_t)std::max(ws->num_sms, 1));
     const size_t off_fcache = round16(off_cache + N * 4);
-    // A call whose trials evaluate more rows than there are feature vectors
-    // evaluates each vector once and looks the others up.  Not into a graph:
-    // it would read the host's copies of the tables when it is replayed.
-    if (mlp_table_wanted(lat, m, nsweeps) && !stream_capturing(stream)) {
-        bool taken = false;
+    // A call of enough unlike trials looks its energies up in a table over all
+    // feature vectors.  Not into a graph: it would read the host's copies of the
+    // tables when it is replayed.
+    if (!call_captured()) {
+        MlpTaken taken;
         st = launch_mlp_table_sweep(lat, m, occ, seed, replica, sweep0, nsweeps, kT, e_acc, n_acc, P.D.df,
-                                    off_fcache + N * 16, &taken, stream);
-        if (st != SMC_OK || taken) return st;
+                                    off_fcache + N * 16, (pl.ntiles + pl.grid - 1) / pl.grid, &taken, &P.route, stream);
+        if (st != SMC_OK || taken == kMlpTabulate) return st;
+        if (taken == kMlpEvaluate) P.route = nullptr;
     }
 
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, off_fcache + N * 16, &st);
@@ -1001,9 +1004,9 @@ smc_status launch_mlp_sweep(const smc_lattice *lat, const smc_model *m, int8_t *
     cudaError_t e = cudaMemsetAsync(scr, 0, off_misc + 16, stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(sweep scratch)");
     st = net ? mlp_energy_launch<NetRelu96>(ws, lat, P.mlpw, occ, P.ecache, P.fcache, (double *)(scr + off_parts),
-                                            P.abort_flag, nullptr, 0, stream)
+                                            P.route, P.abort_flag, nullptr, 0, stream)
              : mlp_energy_launch<NetSilu64>(ws, lat, P.mlpw, occ, P.ecache, P.fcache, (double *)(scr + off_parts),
-                                            P.abort_flag, nullptr, 0, stream);
+                                            P.route, P.abort_flag, nullptr, 0, stream);
     if (st != SMC_OK) return st;
 
     bool constant = true;

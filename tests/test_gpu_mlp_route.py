@@ -1,0 +1,135 @@
+"""MLP sweeps take the faster of their two routes, evaluating the rows of every
+trial or looking f up in a table over all feature vectors, by the box and by the
+share of unlike neighbours that it holds: the same results on either, no host
+wait for the choice, and no call much slower than on the better route."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_2604_08250_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+KT = inputs.K_B_EV * 800.0
+
+
+@pytest.fixture(scope="module")
+def smc():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2604_08250_gb300 import build, smc as s
+    build.build()
+    s.lib()
+    return s
+
+
+def _model(smc, kind, S):
+    if kind == "mlp":
+        return smc.Model(smc.MLP_BF16, mlp=inputs.mlp_weights(3))
+    if kind == "net":
+        return smc.Model(smc.MLPNET_BF16, net=inputs.mlpnet_weights(3))
+    return smc.Model(smc.PAIR_F32_MLP_BF16, 3, inputs.pair_f32_coeffs(5, 3, S), mlp=inputs.mlp_weights(3))
+
+
+def _alloy(smc, dims, fractions, seed=3):
+    lat = smc.Lattice(*dims, len(fractions))
+    counts = (np.array(fractions) * lat.nsites).astype(np.int64)
+    counts[0] += lat.nsites - counts.sum()
+    occ = torch.empty(lat.nsites, dtype=torch.int8, device="cuda")
+    smc.init_lattice(lat, counts, seed, occ)
+    return lat, occ
+
+
+def _sweep(smc, lat, model, occ, n, route=0):
+    occ = occ.clone()
+    e = torch.zeros(1, dtype=torch.float64, device="cuda")
+    a = torch.zeros(1, dtype=torch.int64, device="cuda")
+    smc.debug_set(smc.DBG_MLP_TABLE, route)
+    try:
+        smc.sweep(lat, model, occ, 7, 2, n, KT, e_acc=e, n_acc=a)
+    finally:
+        smc.debug_set(smc.DBG_MLP_TABLE, 0)
+    return occ, e, a
+
+
+# rows of two link cells, of a number that does not fill whole warps, of one warp and of the longest row that fits
+@pytest.mark.parametrize("dims", [(8, 8, 8), (36, 12, 8), (32, 8, 20), (512, 8, 8)])
+@pytest.mark.parametrize("kind", ["mlp", "pair+mlp", "net"])
+@pytest.mark.parametrize("S", [2, 3])
+def test_both_routes_agree(smc, dims, kind, S):
+    lat, occ = _alloy(smc, dims, [1.0 / S] * S)
+    model = _model(smc, kind, S)
+    o1, e1, a1 = _sweep(smc, lat, model, occ, 2, route=1)
+    o2, e2, a2 = _sweep(smc, lat, model, occ, 2, route=2)
+    smc.check()
+    assert not torch.equal(o1, occ) and torch.equal(o1, o2) and int(a1) == int(a2)
+    # the same FP32 dE values summed in FP64 in another order
+    assert abs(float(e1) - float(e2)) <= 1e-12 * lat.nsites
+
+
+# a box whose random alloys are tabulated, and that evaluates where few neighbours are unlike
+FRACTIONS = [[0.2] * 5, [0.99, 0.01, 0.0, 0.0, 0.0], [1.0, 0.0, 0.0, 0.0, 0.0], [0.5, 0.5, 0.0, 0.0, 0.0]]
+
+
+@pytest.mark.parametrize("fractions", FRACTIONS)
+@pytest.mark.parametrize("kind", ["mlp", "net"])
+@pytest.mark.parametrize("busy", [False, True])
+def test_choice_by_the_lattice(smc, fractions, kind, busy):
+    """busy: the stream has work ahead, so that both routes are enqueued before the device has chosen."""
+    lat, occ = _alloy(smc, (96, 96, 96), fractions)
+    model = _model(smc, kind, 5)
+    o1, e1, a1 = _sweep(smc, lat, model, occ, 24, route=1)
+    _sweep(smc, lat, model, occ, 24)  # its buffers
+    torch.cuda.synchronize()
+    got = occ.clone()
+    e = torch.zeros(1, dtype=torch.float64, device="cuda")
+    a = torch.zeros(1, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    if busy:
+        torch.cuda._sleep(1 << 30)  # half a second and more
+    done = torch.cuda.Event()
+    done.record()
+    smc.sweep(lat, model, got, 7, 2, 24, KT, e_acc=e, n_acc=a)
+    assert not busy or not done.query()  # the call came back before the work ahead of it was done
+    smc.check()
+    assert torch.equal(got, o1) and int(a) == int(a1)
+    assert abs(float(e) - float(e1)) <= 1e-12 * lat.nsites * 24
+
+
+def _ms(fn):
+    fn()
+    best = float("inf")
+    for _ in range(3):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        fn()
+        torch.cuda.synchronize()
+        best = min(best, 1e3 * (time.perf_counter() - t))
+    return best
+
+
+# the tabulated route takes 1.3 to 2 times the other's time in the first four, the evaluating one in the others
+@pytest.mark.parametrize("dims,kind,fractions,n", [((128, 128, 128), "mlp", FRACTIONS[1], 12), ((32, 32, 32), "mlp", FRACTIONS[0], 600),
+                                                   ((128, 128, 128), "net", FRACTIONS[1], 6), ((16, 16, 16), "net", FRACTIONS[0], 1000),
+                                                   ((128, 128, 128), "mlp", FRACTIONS[0], 16), ((64, 64, 64), "net", [0.5, 0.5], 20)])
+def test_no_call_is_much_slower_than_on_the_better_route(smc, dims, kind, fractions, n):
+    lat, occ = _alloy(smc, dims, fractions)
+    model = _model(smc, kind, len(fractions))
+    times = [_ms(lambda: _sweep(smc, lat, model, occ, n, route)) for route in (1, 2, 0)]
+    assert times[2] <= 1.2 * min(times[:2]) + 0.2, times
+
+
+def test_occupancy_at_any_address(smc):
+    """The unlike neighbours are counted by words where the occupancy is aligned, by bytes elsewhere."""
+    lat, occ = _alloy(smc, (96, 96, 96), FRACTIONS[1])
+    model = _model(smc, "mlp", 5)
+    want, _, _ = _sweep(smc, lat, model, occ, 24, route=1)
+    for shift in (1, 2):
+        buf = torch.zeros(lat.nsites + 4, dtype=torch.int8, device="cuda")
+        at = buf[shift:shift + lat.nsites]
+        at.copy_(occ)
+        smc.sweep(lat, model, at, 7, 2, 24, KT)
+        smc.check()
+        assert torch.equal(at, want)
