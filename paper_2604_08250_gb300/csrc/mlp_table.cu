@@ -769,16 +769,12 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
                  o_red = up(o_D + kDEntries * 4), o_state = up(o_red + lc_reduce_bytes()),
                  need = std::max(o_state + N * 8, least);
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, need, &st);
-    if (!scr) {  // no room for the table: the evaluating sweep needs none
-        cudaGetLastError();
-        return SMC_OK;
-    }
+    if (!scr) return out_of_memory() ? SMC_OK : st;  // no room beside the table: the evaluating sweep may have it
     void *table = nullptr;
     const size_t table_bytes = up((size_t)T.d.entries * 4);  // then the count and the route word
-    if (table_buffer(table_bytes + 16, &table) != cudaSuccess) {
-        cudaGetLastError();
-        return SMC_OK;
-    }
+    const cudaError_t room = table_buffer(table_bytes + 16, &table);
+    if (room == cudaErrorMemoryAllocation) return SMC_OK;
+    if (room != cudaSuccess) return cuda_fail(room, "cudaMalloc(MLP table)");
     *taken = certain ? kMlpTabulate : kMlpEither;
     P.part_e = (double *)scr;
     P.part_n = (long long *)(scr + o_pn);

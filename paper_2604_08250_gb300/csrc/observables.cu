@@ -444,7 +444,8 @@ smc_status launch_pair_counts(const smc_lattice *lat, int nshells, const int8_t 
         S * (S + 1) / 2 * nshells <= 84) {
         const int nw = lat->nx / 32;
         const long long nwords = rows * nw;
-        uint4 *planes = (uint4 *)planes_buffer(0, (size_t)nwords * sizeof(uint4), stream);
+        uint4 *planes = (uint4 *)planes_buffer(0, (size_t)nwords * sizeof(uint4), &st, stream);
+        if (st != SMC_OK) return st;
         if (planes) {
             launch_planes_aligned(occ, nwords, planes, ws->num_sms, stream);
             if (planes_counts(nshells, S, ws->num_sms * 4, planes, nw, lat->ny, lat->nz, counts, stream)) {

@@ -349,23 +349,28 @@ void own_launch(const Planes &P, int blocks, void *cache, unsigned long long *qu
 
 // The planes' buffer: grown when needed, kept apart from the workspace (whose
 // scratch the callers already use for the counts).  NULL, with nothing
-// changed, without memory or when a captured stream would have to grow it.
+// changed, without memory or when a captured stream would have to grow it
+// (*st = SMC_OK), and on any other error (*st).
 // Graphs may hold the buffer of the pair counts of aligned rows (0), so other
 // calls, never captured, grow one of their own (1).
-void *planes_buffer(int which, size_t bytes, cudaStream_t stream)
+void *planes_buffer(int which, size_t bytes, smc_status *st, cudaStream_t stream)
 {
+    *st = SMC_OK;
     static void *bufs[2];
     static size_t caps[2];
     static int devs[2] = {-1, -1};
     static bool held[2];
     void *&buf = bufs[which];
     int d = 0;
-    if (cudaGetDevice(&d) != cudaSuccess) return nullptr;
-    if (!buf || bytes > caps[which] || d != devs[which]) {
-        if (stream_capturing(stream) || cudaDeviceSynchronize() != cudaSuccess) return nullptr;
+    cudaError_t e = cudaGetDevice(&d);
+    if (e == cudaSuccess && (!buf || bytes > caps[which] || d != devs[which])) {
+        if (stream_capturing(stream)) return nullptr;
         void *p = nullptr;
-        if (device_alloc(&p, bytes) != cudaSuccess) {
-            cudaGetLastError();
+        e = cudaDeviceSynchronize();
+        if (e == cudaSuccess) e = device_alloc(&p, bytes);
+        if (e == cudaErrorMemoryAllocation) return nullptr;
+        if (e != cudaSuccess) {
+            *st = cuda_fail(e, "cudaMalloc(planes)");
             return nullptr;
         }
         release(buf, held[which]);
@@ -373,6 +378,10 @@ void *planes_buffer(int which, size_t bytes, cudaStream_t stream)
         caps[which] = bytes;
         devs[which] = d;
         held[which] = false;
+    }
+    if (e != cudaSuccess) {
+        *st = cuda_fail(e, "cudaGetDevice");
+        return nullptr;
     }
     if (call_captured()) held[which] = true;
     return buf;
@@ -383,12 +392,8 @@ bool planes_build(PlaneLattice lat, int nx, int ny, int nz, const int8_t *occ, i
 {
     *st = SMC_OK;
     if (stream_capturing(stream)) return false;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    if (dev >= 64 || !g_vec_ready[dev]) {
-        *st = vec_tables();
-        if (*st != SMC_OK) return false;
-    }
+    *st = vec_tables();
+    if (*st != SMC_OK) return false;
     P.nx = nx;
     P.ny = ny;
     P.nz = nz;
@@ -396,7 +401,7 @@ bool planes_build(PlaneLattice lat, int nx, int ny, int nz, const int8_t *occ, i
     P.num_sms = num_sms;
     const long long rows = (long long)(lat == kPlanesBcc ? 2 : 4) * ny * nz;
     const int nw = (nx + 31) / 32;
-    uint4 *words = (uint4 *)planes_buffer(1, (size_t)(rows * nw) * sizeof(uint4), stream);
+    uint4 *words = (uint4 *)planes_buffer(1, (size_t)(rows * nw) * sizeof(uint4), st, stream);
     if (!words) return false;
     P.words = words;
     if (nx % 32 == 0 && (uintptr_t)occ % 16 == 0) {

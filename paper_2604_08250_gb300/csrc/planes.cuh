@@ -34,6 +34,6 @@ smc_status planes_own(const Planes &P, int nsh, void *cache, unsigned long long 
 
 // nx % 32 == 0, occ 16-byte aligned (observables.cu).
 void launch_planes_aligned(const int8_t *occ, long long nwords, uint4 *planes, int num_sms, cudaStream_t stream);
-void *planes_buffer(int which, size_t bytes, cudaStream_t stream);
+void *planes_buffer(int which, size_t bytes, smc_status *st, cudaStream_t stream);
 
 }  // namespace smc

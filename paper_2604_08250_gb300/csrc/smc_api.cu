@@ -27,8 +27,13 @@ void set_error(const char *fmt, ...)
     va_end(ap);
 }
 
+static thread_local cudaError_t g_last_error = cudaSuccess;
+
+bool out_of_memory() { return g_last_error == cudaErrorMemoryAllocation; }
+
 smc_status cuda_fail(cudaError_t e, const char *what)
 {
+    g_last_error = e;
     set_error("%s: %s", what, cudaGetErrorString(e));
     return SMC_ERR_CUDA;
 }

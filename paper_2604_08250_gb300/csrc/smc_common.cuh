@@ -141,6 +141,9 @@ __device__ __forceinline__ int ld_volatile_i32(const int *p)
 // ---------------------------------------------------------------------------
 void set_error(const char *fmt, ...);
 smc_status cuda_fail(cudaError_t e, const char *what);
+// Whether the error of this thread's last cuda_fail was a lack of device
+// memory, for which a caller may have a route that needs less.
+bool out_of_memory();
 
 // Per-device workspace (grown with cudaMalloc, never shrunk).
 struct Workspace {

@@ -1215,15 +1215,17 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
         // 140 x 144 x 144 11.4 / 4.2 ms; 160-cell rows no longer fit.
         const int first = res_cols(R, lats, ws->num_sms);
         const int second = first != kResCols ? kResCols : (R == 1 ? kResColsWide : 0);
+        bool no_room = false;
         for (int ncols : {first, second}) {
             if (!ncols) break;
             free_waves(mp);
             st = is_int ? build_res_multi<true>(R, lats, pt, ws, ncols, mp) : build_res_multi<false>(R, lats, pt, ws, ncols, mp);
-            if (R == 1 && ncols == kResColsWide && st != SMC_OK) {  // no room for the lists: the streaming kernels
-                cudaGetLastError();
+            if (R == 1 && ncols == kResColsWide && st != SMC_OK && out_of_memory()) {
+                // no room for the lists now: the streaming kernels, and another look at the next call
                 free_waves(mp);
                 mp.ok = false;
                 st = SMC_OK;
+                no_room = true;
             }
             if (st != SMC_OK || mp.ok) break;
         }
@@ -1233,7 +1235,7 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
             plan_cached.ok = false;
             return st;
         }
-        key_cached = key;
+        if (!no_room) key_cached = key;
     }
     const ResMulti &mp = plan_cached;
     if (!mp.ok) return SMC_ERR_UNSUPPORTED;
@@ -1279,10 +1281,7 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
     const size_t off_exch = off_tab + ((tabs.size() * 4 + 255) / 256) * 256;
     const size_t off_ver = off_exch + exmax;
     unsigned char *scr = (unsigned char *)workspace_scratch(ws, off_ver + vwmax * 8, &st);
-    if (!scr && R == 1 && mp.ncols == kResColsWide) {  // the streaming kernels need less
-        cudaGetLastError();
-        return SMC_ERR_UNSUPPORTED;
-    }
+    if (!scr && R == 1 && mp.ncols == kResColsWide && out_of_memory()) return SMC_ERR_UNSUPPORTED;  // streaming needs less
     if (!scr) return st;
     cudaError_t e = cudaSuccess;
     if (!tabs.empty()) {
