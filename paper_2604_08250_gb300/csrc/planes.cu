@@ -347,44 +347,34 @@ void own_launch(const Planes &P, int blocks, void *cache, unsigned long long *qu
 
 }  // namespace
 
-// The planes' buffer: grown when needed, kept apart from the workspace (whose
-// scratch the callers already use for the counts).  NULL, with nothing
+// The planes' buffer: one per device, grown when needed, kept apart from the
+// workspace's scratch (which the callers already use for the counts).  NULL, with nothing
 // changed, without memory or when a captured stream would have to grow it
 // (*st = SMC_OK), and on any other error (*st).
 // Graphs may hold the buffer of the pair counts of aligned rows (0), so other
 // calls, never captured, grow one of their own (1).
 void *planes_buffer(int which, size_t bytes, smc_status *st, cudaStream_t stream)
 {
-    *st = SMC_OK;
-    static void *bufs[2];
-    static size_t caps[2];
-    static int devs[2] = {-1, -1};
-    static bool held[2];
-    void *&buf = bufs[which];
-    int d = 0;
-    cudaError_t e = cudaGetDevice(&d);
-    if (e == cudaSuccess && (!buf || bytes > caps[which] || d != devs[which])) {
+    Workspace *ws = workspace(st);
+    if (!ws) return nullptr;
+    auto &p = ws->planes[which];
+    if (bytes > p.cap) {
         if (stream_capturing(stream)) return nullptr;
-        void *p = nullptr;
-        e = cudaDeviceSynchronize();
-        if (e == cudaSuccess) e = device_alloc(&p, bytes);
+        void *buf = nullptr;
+        cudaError_t e = cudaDeviceSynchronize();
+        if (e == cudaSuccess) e = device_alloc(&buf, bytes);
         if (e == cudaErrorMemoryAllocation) return nullptr;
         if (e != cudaSuccess) {
             *st = cuda_fail(e, "cudaMalloc(planes)");
             return nullptr;
         }
-        release(buf, held[which]);
-        buf = p;
-        caps[which] = bytes;
-        devs[which] = d;
-        held[which] = false;
+        release(p.buf, p.held);
+        p.buf = buf;
+        p.cap = bytes;
+        p.held = false;
     }
-    if (e != cudaSuccess) {
-        *st = cuda_fail(e, "cudaGetDevice");
-        return nullptr;
-    }
-    if (call_captured()) held[which] = true;
-    return buf;
+    if (call_captured()) p.held = true;
+    return p.buf;
 }
 
 bool planes_build(PlaneLattice lat, int nx, int ny, int nz, const int8_t *occ, int num_sms, Planes &P, smc_status *st,

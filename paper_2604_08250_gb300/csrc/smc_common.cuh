@@ -152,6 +152,11 @@ struct Workspace {
     size_t cap = 0;
     bool held = false;      // a graph may hold buf
     int *status = nullptr;  // latched device status (never moves)
+    struct {
+        void *buf = nullptr;
+        size_t cap = 0;
+        bool held = false;
+    } planes[2];            // neighbour-count planes (planes.cu)
     int num_sms = 0;
     size_t smem_optin = 0;
 };
