@@ -2115,14 +2115,14 @@ static smc_status sweep_impl(int R, const smc_lattice *lats, const smc_model *m,
         st = one_cta(!fast || R >= 16 ? kCtaMaxTrials : 48);
         if (st != SMC_ERR_UNSUPPORTED) return st;
     }
+    // (paired kernel: bulk row copies, so 16-byte aligned rows)
+    const bool wide = fast && fast_wide(R, lats, pt.nsh, pt.sw) && (uintptr_t)occ[0] % 16 == 0;
     if (debug_resident() == 0) {
         // lattices that fit in the SMs' shared memory stay there
-        st = launch_pair_sweep_resident(R, lats, m, pt, occ, seed, replica0, sweep0, nsweeps, kT, e_acc, n_acc,
+        st = launch_pair_sweep_resident(R, lats, m, pt, occ, seed, replica0, sweep0, nsweeps, kT, wide, e_acc, n_acc,
                                         stream);
         if (st != SMC_ERR_UNSUPPORTED) return st;
     }
-    // (paired kernel: bulk row copies, so 16-byte aligned rows)
-    const bool wide = fast && fast_wide(R, lats, pt.nsh, pt.sw) && (uintptr_t)occ[0] % 16 == 0;
     if (cta && !wide) {  // boxes that the resident kernel does not take (two link cells along y or z): 92 against 178 us
         st = one_cta(kCtaMaxTrials);
         if (st != SMC_ERR_UNSUPPORTED) return st;

@@ -44,8 +44,7 @@
 #include <cmath>
 #include <cstring>
 #include <functional>
-#include <map>
-#include <set>
+#include <list>
 #include <vector>
 
 #include "pair_fixed.cuh"
@@ -666,38 +665,36 @@ struct ResPlan {
     const void *kernel = nullptr;
 };
 
-// Rows (sub, y, z) -> id (sub * nz + z) * ny + y read and written by column
-// (cy, cz) in group g (the same sets as the streaming kernel stages).
-void column_rows(int cy, int cz, int g, int ny, int nz, int nsh, std::vector<int> &R, std::vector<int> &W)
+int wrap_row(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }  // v in [-n, 2n)
+
+// Calls f(sub, y, z) for the rows that column (cy, cz) reads in group g (the
+// same sets as the streaming kernel stages), or with writes_only for those it
+// writes.
+template <class F>
+void column_rows(int cy, int cz, int g, int ny, int nz, int nsh, bool writes_only, const F &f)
 {
     const int dy = g & 3, dz = (g >> 2) & 3, sub = g >> 4, soff = sub == 0 ? -1 : 0;
     const int y0 = 4 * cy + dy, z0 = 4 * cz + dz;
-    auto id = [&](int s, int y, int z) {
-        y = ((y % ny) + ny) % ny;
-        z = ((z % nz) + nz) % nz;
-        return (s * nz + z) * ny + y;
-    };
-    R.clear();
-    W.clear();
+    auto row = [&](int s, int y, int z) { f(s, wrap_row(y, ny), wrap_row(z, nz)); };
+    if (writes_only) {
+        row(sub, y0, z0);
+        for (int b = 0; b < 2; ++b)
+            for (int a = 0; a < 2; ++a) row(1 - sub, y0 + soff + a, z0 + soff + b);
+        return;
+    }
     for (int b = -1; b <= 1; ++b)
-        for (int a = -1; a <= 1; ++a) R.push_back(id(sub, y0 + a, z0 + b));
+        for (int a = -1; a <= 1; ++a) row(sub, y0 + a, z0 + b);
     for (int sz = 0; sz < 4; ++sz)
         for (int sy = 0; sy < 4; ++sy) {
             if (nsh < 3 && (sy == 0 || sy == 3) && (sz == 0 || sz == 3)) continue;
-            R.push_back(id(1 - sub, y0 + soff - 1 + sy, z0 + soff - 1 + sz));
+            row(1 - sub, y0 + soff - 1 + sy, z0 + soff - 1 + sz);
         }
-    W.push_back(id(sub, y0, z0));
-    for (int b = 0; b < 2; ++b)
-        for (int a = 0; a < 2; ++a) W.push_back(id(1 - sub, y0 + soff + a, z0 + soff + b));
 }
 
-// Window slot of row r for a block with descriptor dd, or -1 outside.
-int res_slot_of(const int *dd, int r, int ny, int nz, int Wy, int Wz)
+// Window slot of row (s, y, z) for a block with descriptor dd, or -1 outside.
+int res_slot_of(const int *dd, int s, int y, int z, int ny, int nz, int Wy, int Wz)
 {
-    const int s = r / (ny * nz), z = (r / ny) % nz, y = r % ny;
-    int yy = y - dd[4 + s], zz = z - dd[6 + s];
-    yy = ((yy % ny) + ny) % ny;
-    zz = ((zz % nz) + nz) % nz;
+    const int yy = wrap_row(y - dd[4 + s], ny), zz = wrap_row(z - dd[6 + s], nz);  // windows start at -2 .. ny - 2
     if (yy >= Wy || zz >= Wz) return -1;
     return (s * Wz + zz) * Wy + yy;
 }
@@ -803,31 +800,50 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
     rp.Wy = res_wy(by, ncols);
     rp.Wz = 4 * bz + 7;
     rp.rowB = rowB;
+    // whether it fits, at the short pitch, is seen as soon as it can be: by the rows alone, then by each block's lists
+    const int nk = (nx / 4 + 31) / 32, short_rowB = (nx + 32 + 15) / 16 * 16;  // (the exchange moves 8 and 16 bytes)
+    auto smem_of = [&](int pitch) {
+        return (size_t)kQRows * pt.rw * 4 + 64 + (size_t)2 * rp.Wy * rp.Wz * pitch +
+               ((size_t)rp.blob * 4 + 15) / 16 * 16 + (size_t)ncols * nk * 512;
+    };
+    if (smem_of(short_rowB) > dyn_max) return SMC_OK;
     const int nrows_lat = 2 * ny * nz;
     auto block_of = [&](int cy, int cz) { return (cz / bz) * rp.NBy + (cy / by); };
-    // per row: writer block at every group (-1 = none)
-    std::vector<int> wblk((size_t)nrows_lat * 32, -1);
-    std::vector<int> R, W;
-    for (int g = 0; g < 32; ++g)
-        for (int cz = 0; cz < NLz; ++cz)
-            for (int cy = 0; cy < NLy; ++cy) {
-                column_rows(cy, cz, g, ny, nz, nsh, R, W);
-                for (int r : W) wblk[(size_t)r * 32 + g] = block_of(cy, cz);
-            }
-    // last write of row r before group g (cyclic over the sweep): writer
-    // block and distance d in groups (1..32), or (-1, 0) if never written
+    auto id = [&](int s, int y, int z) { return (s * nz + z) * ny + y; };
+    // per row: the groups that write it (bit g) and the block that does in each
+    std::vector<uint32_t> wmask((size_t)nrows_lat, 0u);
+    std::vector<uint16_t> wblk((size_t)nrows_lat * 32);
+    for (int cz = 0; cz < NLz; ++cz)
+        for (int cy = 0; cy < NLy; ++cy)
+            for (int g = 0; g < 32; ++g)
+                column_rows(cy, cz, g, ny, nz, nsh, true, [&](int s, int y, int z) {
+                    const int r = id(s, y, z);
+                    wmask[r] |= 1u << g;
+                    wblk[(size_t)r * 32 + g] = (uint16_t)block_of(cy, cz);
+                });
+    // groups as seen from g: bit 32 - d of before(m, g) is group g - d (cyclic over the sweep), d = 1 .. 32
+    auto before = [](uint32_t m, int g) { return (g & 31) ? (m >> (g & 31) | m << (32 - (g & 31))) : m; };
+    // last write of row r before group g: writer block and distance d in groups, or (-1, 0) if never written
     auto last_write = [&](int r, int g, int &d) {
-        for (d = 1; d <= 32; ++d) {
-            const int b = wblk[(size_t)r * 32 + ((g - d + 64) & 31)];
-            if (b >= 0) return b;
-        }
-        d = 0;
-        return -1;
+        const uint32_t m = before(wmask[r], g);
+        d = m ? __builtin_clz(m) + 1 : 0;
+        return m ? (int)wblk[(size_t)r * 32 + ((g - d + 64) & 31)] : -1;
     };
+    std::vector<std::vector<int>> last_rows(rp.nblocks);  // rows whose last write in the sweep is the block's
+    for (int r = 0; r < nrows_lat; ++r) {
+        int d = 0;
+        const int b = last_write(r, 32, d);
+        if (b >= 0) last_rows[b].push_back(r);
+    }
     rp.desc.assign((size_t)rp.nblocks * kResDesc, 0);
     rp.lists.clear();
     const int nc = ncols;  // compute warps of the kernel (some idle for smaller blocks)
-    std::vector<int> vslot((size_t)32 * nrows_lat, -1);  // (group of the write, row) -> version slot
+    std::vector<int> vslot((size_t)32 * nrows_lat, -1);  // (row, group of the write) -> version slot
+    const int nslots = 2 * rp.Wy * rp.Wz;
+    std::vector<uint32_t> rmask(nslots);           // per window row: the groups that read it
+    std::vector<std::pair<int, int>> rows;         // the window rows that are read: (row, slot), by row
+    std::vector<std::vector<std::pair<int, int>>> reads(32);
+    std::vector<std::vector<uint32_t>> ents(33);  // fetch entries of a group by distance
     int nver = 0;
     struct Blk {
         std::vector<uint32_t> hdr, body;
@@ -852,20 +868,24 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
         dd[13] = rp.NBz;
         dd[15] = rp.Wy;
         dd[16] = rp.Wz;
-        // rows the block reads in each group
-        std::vector<std::vector<int>> reads(32);
-        for (int g = 0; g < 32; ++g) {
-            for (int k = 0; k < ncy * ncz; ++k) {
-                column_rows(cy0 + k % ncy, cz0 + k / ncy, g, ny, nz, nsh, R, W);
-                reads[g].insert(reads[g].end(), R.begin(), R.end());
-            }
-            std::sort(reads[g].begin(), reads[g].end());
-            reads[g].erase(std::unique(reads[g].begin(), reads[g].end()), reads[g].end());
-        }
-        auto reads_at = [&](int g, int r) {
-            const auto &v = reads[(g + 64) & 31];
-            return std::binary_search(v.begin(), v.end(), r);
-        };
+        // rows the block reads in each group, by row
+        std::fill(rmask.begin(), rmask.end(), 0u);
+        rows.clear();
+        for (int k = 0; k < ncy * ncz; ++k)
+            for (int g = 0; g < 32; ++g)
+                column_rows(cy0 + k % ncy, cz0 + k / ncy, g, ny, nz, nsh, false, [&](int s, int y, int z) {
+                    const int sl = res_slot_of(dd, s, y, z, ny, nz, rp.Wy, rp.Wz);
+                    if (sl < 0) {
+                        fits = false;
+                        return;
+                    }
+                    if (rmask[sl] == 0u) rows.push_back({id(s, y, z), sl});
+                    rmask[sl] |= 1u << g;
+                });
+        std::sort(rows.begin(), rows.end());
+        for (auto &v : reads) v.clear();
+        for (const auto &rs : rows)
+            for (uint32_t m = rmask[rs.second]; m; m &= m - 1) reads[__builtin_ctz(m)].push_back(rs);
         Blk &B = blks[blk];
         B.hdr.assign(33 + 32 * nc + 3, 0);  // an even size: the entry pairs stay 8-byte aligned
         // fetch lists per group: rows read at g whose last write is another
@@ -873,34 +893,27 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
         // keeps it): {smem slot | d << 16, version slot}
         for (int g = 0; g < 32; ++g) {
             B.hdr[g] = (uint32_t)(B.hdr.size() + B.body.size());
-            std::vector<std::pair<int, std::pair<uint32_t, uint32_t>>> ents;  // (-d, entry)
-            for (int r : reads[g]) {
+            for (auto &v : ents) v.clear();
+            for (const auto &rs : reads[g]) {
+                const int r = rs.first, sl = rs.second;
                 int d = 0;
                 const int wb = last_write(r, g, d);
                 if (wb < 0 || wb == blk) continue;
-                bool seen = false;
-                for (int h = g - d + 1; h < g && !seen; ++h) seen = reads_at(h, r);
-                if (seen) continue;
-                const int sl = res_slot_of(dd, r, ny, nz, rp.Wy, rp.Wz);
-                if (sl < 0) {
-                    fits = false;
-                    continue;
-                }
-                int &v = vslot[(size_t)((g - d + 64) & 31) * nrows_lat + r];
+                // read since, in groups g - d + 1 .. g - 1?
+                if (d > 1 && (before(rmask[sl], g) & (~0u << (33 - d)))) continue;
+                int &v = vslot[(size_t)r * 32 + ((g - d + 64) & 31)];
                 if (v < 0) v = nver++;
-                ents.push_back({-d, {(uint32_t)sl | ((uint32_t)d << 16), (uint32_t)v}});
+                ents[d].push_back((uint32_t)sl | ((uint32_t)d << 16));
+                ents[d].push_back((uint32_t)v);
             }
             // oldest versions first: they are ready at once, and the rows
             // written in the previous group (the ones that may still have to
             // be waited for) come last, in as few polling rounds as possible
-            std::stable_sort(ents.begin(), ents.end(),
-                             [](const auto &a, const auto &b) { return a.first < b.first; });
-            for (const auto &en : ents) {
-                B.body.push_back(en.second.first);
-                B.body.push_back(en.second.second);
-            }
+            for (int d = 32; d >= 1; --d) B.body.insert(B.body.end(), ents[d].begin(), ents[d].end());
         }
         B.hdr[32] = (uint32_t)(B.hdr.size() + B.body.size());
+        rp.blob = std::max(rp.blob, (int)(B.hdr.size() + B.body.size() + last_rows[blk].size()));
+        if (smem_of(short_rowB) > dyn_max) return SMC_OK;  // 160^3 and other lattices that stream all the same
     }
     // publish lists per (group, compute warp): the rows a column writes whose
     // version another block reads ({smem slot, version slot}); final rows:
@@ -913,29 +926,23 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
             for (int k = 0; k < nc; ++k) {
                 B.hdr[33 + g * nc + k] = (uint32_t)(B.hdr.size() + B.body.size());
                 if (k >= ncy * ncz) continue;
-                column_rows(cy0 + k % ncy, cz0 + k / ncy, g, ny, nz, nsh, R, W);
-                for (int r : W) {
-                    const int v = vslot[(size_t)g * nrows_lat + r];
-                    if (v < 0) continue;
-                    const int sl = res_slot_of(dd, r, ny, nz, rp.Wy, rp.Wz);
+                column_rows(cy0 + k % ncy, cz0 + k / ncy, g, ny, nz, nsh, true, [&](int s, int y, int z) {
+                    const int v = vslot[(size_t)id(s, y, z) * 32 + g];
+                    if (v < 0) return;
+                    const int sl = res_slot_of(dd, s, y, z, ny, nz, rp.Wy, rp.Wz);
                     if (sl < 0) fits = false;
                     B.body.push_back((uint32_t)sl);
                     B.body.push_back((uint32_t)v);
-                }
+                });
             }
         B.hdr[33 + 32 * nc] = (uint32_t)(B.hdr.size() + B.body.size());
         B.hdr[33 + 32 * nc + 1] = (uint32_t)(B.hdr.size() + B.body.size());
-        uint32_t nfin = 0;
-        for (int r = 0; r < nrows_lat; ++r) {
-            int d = 0;
-            if (last_write(r, 32, d) == blk) {
-                const int sl = res_slot_of(dd, r, ny, nz, rp.Wy, rp.Wz);
-                if (sl < 0) fits = false;
-                B.body.push_back(((uint32_t)sl << 21) | (uint32_t)r);
-                ++nfin;
-            }
+        for (int r : last_rows[blk]) {
+            const int sl = res_slot_of(dd, r / (ny * nz), r % ny, r / ny % nz, ny, nz, rp.Wy, rp.Wz);
+            if (sl < 0) fits = false;
+            B.body.push_back(((uint32_t)sl << 21) | (uint32_t)r);
         }
-        B.hdr[33 + 32 * nc + 2] = nfin;
+        B.hdr[33 + 32 * nc + 2] = (uint32_t)last_rows[blk].size();
         rp.desc[(size_t)blk * kResDesc + 8] = (int)rp.lists.size();
         rp.desc[(size_t)blk * kResDesc + 9] = (int)(B.hdr.size() + B.body.size());
         rp.blob = std::max(rp.blob, (int)(B.hdr.size() + B.body.size()));
@@ -945,12 +952,7 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
     }
     if (!fits) return SMC_OK;  // a row outside the window (not expected)
     rp.nver = std::max(nver, 1);
-    const int nk = (nx / 4 + 31) / 32;
-    auto smem_of = [&](int pitch) {
-        return (size_t)kQRows * pt.rw * 4 + 64 + (size_t)2 * rp.Wy * rp.Wz * pitch +
-               ((size_t)rp.blob * 4 + 15) / 16 * 16 + (size_t)nc * nk * 512;
-    };
-    if (smem_of(rowB) > dyn_max) rowB = (nx + 32 + 15) / 16 * 16;  // (the exchange moves 8 and 16 bytes)
+    if (smem_of(rowB) > dyn_max) rowB = short_rowB;
     rp.rowB = rowB;
     const size_t smem = smem_of(rowB);
     if (smem > dyn_max) return SMC_OK;
@@ -1185,7 +1187,7 @@ smc_status build_res_multi(int R, const smc_lattice *lats, const PairTable &pt, 
 
 smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_model *m, const PairTable &pt,
                                       int8_t *const *occ, uint64_t seed, uint32_t replica0, uint64_t sweep0,
-                                      int nsweeps, const double *kT, double *e_acc, int64_t *n_acc,
+                                      int nsweeps, const double *kT, bool paired, double *e_acc, int64_t *n_acc,
                                       cudaStream_t stream)
 {
     if (R < 1 || R > kMaxReplicas) return SMC_ERR_UNSUPPORTED;
@@ -1199,15 +1201,32 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
     Workspace *ws = workspace(&st);
     if (!ws) return st;
     const bool is_int = m->kind == SMC_PAIR_I32;
-    static std::vector<long long> key_cached;
-    static ResMulti plan_cached;
+    // A lattice that only wide blocks hold, for a call of few sweeps: filling and emptying the blocks costs more than
+    // streaming.  Resident / streaming, ms: 128 x 160 x 160, whose streaming kernel pairs its groups, 1 sweep
+    // 0.33 / 0.22, 3 sweeps 0.59 / 0.56, 5 sweeps 0.84 / 0.88; one sweep of 64 x 192 x 192 0.38 / 0.32, of
+    // 64 x 160 x 160 0.31 / 0.32 and with three shells 0.38 / 0.35, of rows that are no multiple of 16 cells
+    // (140 x 144 x 144) 0.40 / 0.62.
+    const bool one = nsweeps == 1 && lats[0].nx % 16 == 0 && (pt.nsh >= 3 || lats[0].ny / 4 * (lats[0].nz / 4) > 1800);
+    if (R == 1 && (paired ? nsweeps < 5 : one)) {
+        int by = 0, bz = 0;
+        if (!res_shape(lats[0], ws->num_sms, false, kResCols, by, bz)) return SMC_ERR_UNSUPPORTED;
+    }
+    // the plans of the last lattices, the latest first (programs take turns with a few): making one takes 9 ms for
+    // 64 x 160 x 160 cells (57 ms with the sets and sorts of every group), 6 ms for 64 x 128 x 128 (38 ms)
+    struct PlanEntry {
+        std::vector<long long> key;
+        ResMulti plan;
+    };
+    static std::list<PlanEntry> plans;
+    constexpr size_t kPlans = 4;
     const Tuning tu = current_tuning();
     std::vector<long long> key = {R, pt.nsh, pt.sw, is_int, ws->device, ws->num_sms, tu.tile_y, tu.tile_z};
     for (int r = 0; r < R; ++r) key.insert(key.end(), {lats[r].nx, lats[r].ny, lats[r].nz});
-    if (key != key_cached) {
-        if (stream_capturing(stream)) return SMC_ERR_UNSUPPORTED;  // a plan's lists cannot be allocated into a graph
-        free_waves(plan_cached);
-        key_cached.clear();
+    auto known = std::find_if(plans.begin(), plans.end(), [&](const PlanEntry &p) { return p.key == key; });
+    if (known != plans.end()) {
+        plans.splice(plans.begin(), plans, known);
+    } else {
+        if (call_captured()) return SMC_ERR_UNSUPPORTED;  // a plan's lists cannot be allocated into a graph
         ResMulti mp;
         // Wide blocks that do not fit after all: the others.  One lattice with more columns than 152 blocks of 8 hold
         // (up to 2,432 short rows): wide ones.  20 sweeps, streaming / resident: 64 x 160 x 160 5.4 / 2.3 ms, three
@@ -1215,31 +1234,27 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
         // 140 x 144 x 144 11.4 / 4.2 ms; 160-cell rows no longer fit.
         const int first = res_cols(R, lats, ws->num_sms);
         const int second = first != kResCols ? kResCols : (R == 1 ? kResColsWide : 0);
-        bool no_room = false;
         for (int ncols : {first, second}) {
             if (!ncols) break;
             free_waves(mp);
             st = is_int ? build_res_multi<true>(R, lats, pt, ws, ncols, mp) : build_res_multi<false>(R, lats, pt, ws, ncols, mp);
-            if (R == 1 && ncols == kResColsWide && st != SMC_OK && out_of_memory()) {
-                // no room for the lists now: the streaming kernels, and another look at the next call
+            if (st != SMC_OK) {
                 free_waves(mp);
-                mp.ok = false;
-                st = SMC_OK;
-                no_room = true;
+                // no room for the lists now: the streaming kernels, and another look at the next call
+                if (R == 1 && ncols == kResColsWide && out_of_memory()) return SMC_ERR_UNSUPPORTED;
+                return st;
             }
-            if (st != SMC_OK || mp.ok) break;
+            if (mp.ok) break;
         }
-        plan_cached = std::move(mp);
-        if (st != SMC_OK) {
-            free_waves(plan_cached);
-            plan_cached.ok = false;
-            return st;
+        while (plans.size() >= kPlans) {
+            free_waves(plans.back().plan);
+            plans.pop_back();
         }
-        if (!no_room) key_cached = key;
+        plans.push_front({std::move(key), std::move(mp)});
     }
-    const ResMulti &mp = plan_cached;
+    ResMulti &mp = plans.front().plan;
     if (!mp.ok) return SMC_ERR_UNSUPPORTED;
-    if (call_captured()) plan_cached.held = true;
+    if (call_captured()) mp.held = true;
 
     // per-sweep temperatures: one launch per kMaxBeta / (replicas of the wave) sweeps
     bool constant = true;

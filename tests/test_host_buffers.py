@@ -62,3 +62,45 @@ for d in (0, 1) * 4:
     box.sro()
 assert counts() == before, (before, counts())
 """)
+
+
+def test_lattices_in_turn_keep_their_plans(run):
+    """Resident plans (one with columns for wide blocks only): made once for each of a few lattices."""
+    run("""
+m = model()
+boxes = [Box(64, 64, 64), Box(64, 160, 160), Box(48, 48, 48)]
+for b in boxes:
+    b.sweep(m, 20)
+before = counts()
+for b in boxes * 3:
+    b.sweep(m, 20)
+assert counts() == before, (before, counts())
+""")
+
+
+def test_old_plans_are_given_back(run):
+    run("""
+m = model()
+Box(96, 96, 96).sweep(m, 20)  # the largest: the workspace does not grow any more
+start = counts()
+for e in range(24, 64, 4):
+    Box(e, e, e).sweep(m, 20)
+made, freed, _ = [b - a for a, b in zip(start, counts())]
+assert made == 10 and made - freed <= 3, (made, freed)
+""")
+
+
+def test_a_lattice_that_streams_makes_no_lists(run):
+    run("""
+import time
+m = model()
+Box(24, 24, 24).sweep(m, 20)
+def first(box, n):
+    t = time.perf_counter()
+    box.sweep(m, n)
+    return time.perf_counter() - t
+plan = first(Box(64, 160, 160), 20)
+# rows too long for wide blocks; one sweep of a lattice that streams faster
+for box, n in ((Box(192, 160, 160), 20), (Box(128, 160, 152), 1)):
+    assert first(box, n) < 0.2 * plan
+""")
