@@ -912,7 +912,10 @@ smc_status build_res_plan(const smc_lattice &lat, const PairTable &pt, Workspace
             for (int d = 32; d >= 1; --d) B.body.insert(B.body.end(), ents[d].begin(), ents[d].end());
         }
         B.hdr[32] = (uint32_t)(B.hdr.size() + B.body.size());
-        rp.blob = std::max(rp.blob, (int)(B.hdr.size() + B.body.size() + last_rows[blk].size()));
+        // its lists so far, its final rows, and, where all blocks are equal, its published versions: as many as all
+        // blocks fetch, each version by at most three (a row lies in two blocks' windows along each axis)
+        const bool equal = NLy % by == 0 && NLz % bz == 0;
+        rp.blob = std::max(rp.blob, (int)(B.hdr.size() + B.body.size() * (equal ? 4 : 3) / 3 + last_rows[blk].size()));
         if (smem_of(short_rowB) > dyn_max) return SMC_OK;  // 160^3 and other lattices that stream all the same
     }
     // publish lists per (group, compute warp): the rows a column writes whose

@@ -101,6 +101,6 @@ def first(box, n):
     return time.perf_counter() - t
 plan = first(Box(64, 160, 160), 20)
 # rows too long for wide blocks; one sweep of a lattice that streams faster
-for box, n in ((Box(192, 160, 160), 20), (Box(128, 160, 152), 1)):
+for box, n in ((Box(160, 160, 160), 20), (Box(192, 160, 160), 20), (Box(128, 160, 152), 1)):
     assert first(box, n) < 0.2 * plan
 """)
