@@ -228,6 +228,8 @@ smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_
                                       int8_t *const *occ, uint64_t seed, uint32_t replica0, uint64_t sweep0,
                                       int nsweeps, const double *kT, bool paired, double *e_acc, int64_t *n_acc,
                                       cudaStream_t stream);
+// Launches per call that the resident sweep of R replicas takes (0: it has no block shape for one).
+int resident_waves(int R, const smc_lattice *lats, int num_sms);
 int debug_resident();
 
 // The sweep of small boxes by one CTA per replica (sweep_cta.cu):

@@ -2102,17 +2102,20 @@ static smc_status sweep_impl(int R, const smc_lattice *lats, const smc_model *m,
     // Small boxes run in one CTA each (sweep_cta.cu), boxes whose rows fit the
     // SMs' shared memory resident there (sweep_resident.cu).  Measured per sweep
     // (two shells, FP32): 8^3 cells 38 us in one CTA against 165 streaming; 12^3
-    // 48 against 60 resident, 16^3 61 and 62, 20^3 93 and 63; sixty-four 20^3
-    // replicas 100 against 304 (the resident kernel takes them in waves); boxes
-    // with an axis that is no multiple of four, one trial per mini-step along
-    // it, 8 to 20 times less than the general kernel.
+    // 48 against 60 resident, 16^3 61 and 62, 20^3 93 and 63; boxes with an axis
+    // that is no multiple of four, one trial per mini-step along it, 8 to 20
+    // times less than the general kernel.  Replicas take one CTA each at the
+    // same time, but share resident launches only as far as their blocks fit the
+    // SMs: 20^3, 16 replicas 102 us in a CTA each against 79 in one wave of
+    // resident blocks, 17 replicas 102 against 145 in two, 64 replicas 104 against
+    // 309 in four; 16^3, 9 replicas 63 against 76, 10 replicas 63 against 141.
     const bool cta = debug_resident() == 0 && debug_skip_tile() < 0;
     auto one_cta = [&](int most) {
         return launch_pair_sweep_cta(R, lats, m, pt, occ, seed, replica0, sweep0, nsweeps, kT, most, fast, e_acc, n_acc,
                                      stream);
     };
     if (cta) {
-        st = one_cta(!fast || R >= 16 ? kCtaMaxTrials : 48);
+        st = one_cta(!fast || (R > 1 && resident_waves(R, lats, ws->num_sms) > 1) ? kCtaMaxTrials : (R > 1 ? 64 : 48));
         if (st != SMC_ERR_UNSUPPORTED) return st;
     }
     // (paired kernel: bulk row copies, so 16-byte aligned rows)

@@ -1026,6 +1026,26 @@ void free_waves(ResMulti &mp)
     mp.held = false;
 }
 
+// Launches that R replicas in blocks of up to ncols columns share, first fit
+// decreasing as the waves are filled; 0 when one has no block shape.
+int res_waves(int R, const smc_lattice *lats, int num_sms, int ncols)
+{
+    std::vector<int> nb, bins;
+    for (int r = 0; r < R; ++r) {
+        int by = 0, bz = 0;
+        if (!res_shape(lats[r], num_sms, true, ncols, by, bz) || (ncols != kResCols && lats[r].nx > kResWideRow)) return 0;
+        nb.push_back(((lats[r].ny / 4 + by - 1) / by) * ((lats[r].nz / 4 + bz - 1) / bz));
+    }
+    std::sort(nb.begin(), nb.end(), std::greater<int>());
+    for (int n : nb) {
+        size_t i = 0;
+        while (i < bins.size() && bins[i] + n > num_sms) ++i;
+        if (i == bins.size()) bins.push_back(0);
+        bins[i] += n;
+    }
+    return (int)bins.size();
+}
+
 // Compute warps per CTA for R replicas.  A wave's time is its groups', 2.77 us
 // each with 8 warps, 3.6 us with 16 (bound by issue then, where 8 leave the
 // schedulers waiting for each other's rows half of the time), so wide blocks
@@ -1036,25 +1056,8 @@ int res_cols(int R, const smc_lattice *lats, int num_sms)
 {
     const Tuning tu = current_tuning();
     if (R < 2 || (tu.tile_y > 0 && tu.tile_z > 0)) return kResCols;
-    int waves[2] = {0, 0};
-    for (int wide = 0; wide < 2; ++wide) {
-        std::vector<int> nb, bins;
-        for (int r = 0; r < R; ++r) {
-            int by = 0, bz = 0;
-            if (!res_shape(lats[r], num_sms, true, wide ? kResColsWide : kResCols, by, bz)) return kResCols;
-            if (wide && lats[r].nx > kResWideRow) return kResCols;
-            nb.push_back(((lats[r].ny / 4 + by - 1) / by) * ((lats[r].nz / 4 + bz - 1) / bz));
-        }
-        std::sort(nb.begin(), nb.end(), std::greater<int>());
-        for (int n : nb) {  // first fit, as the waves are filled
-            size_t i = 0;
-            while (i < bins.size() && bins[i] + n > num_sms) ++i;
-            if (i == bins.size()) bins.push_back(0);
-            bins[i] += n;
-        }
-        waves[wide] = (int)bins.size();
-    }
-    return waves[1] * kResWideCost < waves[0] ? kResColsWide : kResCols;
+    const int narrow = res_waves(R, lats, num_sms, kResCols), wide = res_waves(R, lats, num_sms, kResColsWide);
+    return narrow && wide && wide * kResWideCost < narrow ? kResColsWide : kResCols;
 }
 
 template <bool IS_INT>
@@ -1187,6 +1190,11 @@ smc_status build_res_multi(int R, const smc_lattice *lats, const PairTable &pt, 
 }
 
 }  // namespace
+
+int resident_waves(int R, const smc_lattice *lats, int num_sms)
+{
+    return res_waves(R, lats, num_sms, res_cols(R, lats, num_sms));
+}
 
 smc_status launch_pair_sweep_resident(int R, const smc_lattice *lats, const smc_model *m, const PairTable &pt,
                                       int8_t *const *occ, uint64_t seed, uint32_t replica0, uint64_t sweep0,
