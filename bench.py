@@ -36,14 +36,14 @@ BYTES_PER_ATTEMPT = 24.0  # 22 B read set + 2 B written per trial (two-shell pai
 # MLPNet (20 -> 96 -> 96 -> 96 -> 1): 2 (20 96 + 96 96 + 96 96 + 96) FLOP per
 # site evaluation, 40 post-swap evaluations per attempt (pre-swap energies cached)
 NET_FLOP_PER_SITE = 2 * (20 * 96 + 96 * 96 + 96 * 96 + 96)
-NET_FLOP_PER_ATTEMPT = 40 * NET_FLOP_PER_SITE
 QSRO_SEED, QSRO_SHELLS = 7, 2  # qSRO workload parameters
 # zone sites of a qSRO trial besides a and b (within the model's shells of
 # either), counted from the BCC geometry
 QSRO_ZONE = {1: 14, 2: 20, 3: 38}
 MLP_FLOP_PER_SITE_FWD = 2 * (20 * 64 + 64 * 64)  # 10752
 MLP_FLOP_PER_SITE_GRAD = MLP_FLOP_PER_SITE_FWD + 2 * 64 * 64 + 2 * 64 * 64 + 2 * 20 * 64  # 29696
-MLP_FLOP_PER_ATTEMPT = 40 * MLP_FLOP_PER_SITE_FWD  # post-swap energies of the 40-site zone (cached pre-swap)
+# feature vectors of S species: S and the ways to fill 8, 6 and 12 neighbours
+FEATURE_VECTORS = {S: S * math.comb(7 + S, S - 1) * math.comb(5 + S, S - 1) * math.comb(11 + S, S - 1) for S in range(2, 6)}
 
 
 def peaks():
@@ -625,41 +625,44 @@ def run_extras(smc, torch, dev, pk):
     smc.init_lattice(lat4, inputs.dirichlet_counts(lat4.nsites, S, c4["comp_seed"]), c4["mc_seed"], occ4)
     mlp_model = smc.Model(smc.MLP_BF16, mlp=inputs.mlp_weights(c4["mlp_seed"]))
     kT4 = inputs.K_B_EV * c4["T"]
-    n_acc = torch.zeros(1, dtype=torch.int64, device=dev)
     nsw4 = 2
-    f0 = unlike_fraction(lat4, occ4)
-    ms4 = timed(lambda: smc.sweep(lat4, mlp_model, occ4, c4["mc_seed"], 0, nsw4, kT4, n_acc=n_acc), reps=1)
-    fev = 0.5 * (f0 + unlike_fraction(lat4, occ4))
-    att4 = lat4.nsites * nsw4 / (ms4 * 1e-3)
-    acc_rate = float(n_acc.item()) / (2 * lat4.nsites * nsw4)  # warm-up call + timed call
-    tfl = att4 * fev * MLP_FLOP_PER_ATTEMPT / 1e12
-    out["mlp_256"] = {"cells": [n4] * 3, "sweeps_per_launch": nsw4, "ms_per_sweep": ms4 / nsw4,
-                      "attempts_per_s": att4, "job_s_200_sweeps": ms4 / nsw4 * c4["nsweeps"] / 1e3,
-                      "accept_rate": acc_rate, "evaluated_fraction": fev, "achieved_tflops": tfl,
-                      "achieved_tflops_if_every_attempt": att4 * MLP_FLOP_PER_ATTEMPT / 1e12,
-                      "frac_of_measured_bf16_sustained": tfl / pk["bf16_tflops_sustained"],
-                      "flop_per_evaluated_attempt": MLP_FLOP_PER_ATTEMPT,
-                      "note": "attempts with equal species (dE = 0) are not evaluated; evaluated_fraction is the "
-                              "unlike first-shell bond fraction before and after the timed sweeps; a call of this "
-                              "size evaluates every feature vector once and looks f up, so the TFLOP/s count "
-                              "evaluations that are replaced by look-ups"}
+
+    def network_leg(model, flop_per_row):
+        """A call that looks f up evaluates every feature vector once, so these rows are the ones that its TFLOP/s
+        count; the evaluating route (40 rows for each attempt of unlike species) is timed beside it."""
+        n = torch.zeros(1, dtype=torch.int64, device=dev)
+        start = occ4.clone()
+
+        def call(route, occ, n_acc=None):
+            smc.debug_set(smc.DBG_MLP_TABLE, route)
+            smc.sweep(lat4, model, occ, c4["mc_seed"], 0, nsw4, kT4, n_acc=n_acc)
+            smc.debug_set(smc.DBG_MLP_TABLE, 0)
+        ms_eval = timed(lambda: call(1, start), reps=1)
+        f_eval = unlike_fraction(lat4, start)
+        f0 = unlike_fraction(lat4, occ4)
+        ms = timed(lambda: call(2, occ4, n), reps=1)
+        att = lat4.nsites * nsw4
+        rows = FEATURE_VECTORS[S]
+        tf = rows * flop_per_row / (ms * 1e-3) / 1e12
+        tf_eval = att * f_eval * 40 * flop_per_row / (ms_eval * 1e-3) / 1e12
+        return {"cells": [n4] * 3, "sweeps_per_launch": nsw4, "ms_per_sweep": ms / nsw4, "attempts_per_s": att / (ms * 1e-3),
+                "accept_rate": float(n.item()) / (2 * att),  # warm-up call + timed call
+                "unlike_fraction": 0.5 * (f0 + unlike_fraction(lat4, occ4)), "evaluated_rows_per_call": rows,
+                "achieved_tflops": tf, "frac_of_measured_bf16_sustained": tf / pk["bf16_tflops_sustained"],
+                "flop_per_row": flop_per_row,
+                "evaluating_route": {"ms_per_sweep": ms_eval / nsw4, "achieved_tflops": tf_eval,
+                                     "frac_of_measured_bf16_sustained": tf_eval / pk["bf16_tflops_sustained"],
+                                     "unlike_fraction_after": f_eval},
+                "note": "f is evaluated once per feature vector and looked up; attempts with equal species (dE = 0) "
+                        "look nothing up"}
+    out["mlp_256"] = network_leg(mlp_model, MLP_FLOP_PER_SITE_FWD)
+    out["mlp_256"]["job_s_200_sweeps"] = out["mlp_256"]["ms_per_sweep"] * c4["nsweeps"] / 1e3
     e4 = torch.zeros(1, dtype=torch.float64, device=dev)
     ems = timed(lambda: smc.energy(lat4, mlp_model, occ4, e4), reps=3)
     out["mlp_energy_256"] = {"ms": ems, "achieved_tflops": lat4.nsites * MLP_FLOP_PER_SITE_FWD / (ems * 1e-3) / 1e12}
     # MLPNet at the paper's shape on the same lattice and temperature
     net_model = smc.Model(smc.MLPNET_BF16, net=inputs.mlpnet_weights(c4["mlp_seed"]))
-    n_accn = torch.zeros(1, dtype=torch.int64, device=dev)
-    f0 = unlike_fraction(lat4, occ4)
-    msn = timed(lambda: smc.sweep(lat4, net_model, occ4, c4["mc_seed"], 0, nsw4, kT4, n_acc=n_accn), reps=1)
-    fevn = 0.5 * (f0 + unlike_fraction(lat4, occ4))
-    attn = lat4.nsites * nsw4 / (msn * 1e-3)
-    tfn = attn * fevn * NET_FLOP_PER_ATTEMPT / 1e12
-    out["mlpnet_256"] = {"cells": [n4] * 3, "sweeps_per_launch": nsw4, "ms_per_sweep": msn / nsw4,
-                         "attempts_per_s": attn, "accept_rate": float(n_accn.item()) / (2 * lat4.nsites * nsw4),
-                         "evaluated_fraction": fevn, "achieved_tflops": tfn,
-                         "achieved_tflops_if_every_attempt": attn * NET_FLOP_PER_ATTEMPT / 1e12,
-                         "frac_of_measured_bf16_sustained": tfn / pk["bf16_tflops_sustained"],
-                         "flop_per_evaluated_attempt": NET_FLOP_PER_ATTEMPT}
+    out["mlpnet_256"] = network_leg(net_model, NET_FLOP_PER_SITE)
     en = torch.zeros(1, dtype=torch.float64, device=dev)
     emsn = timed(lambda: smc.energy(lat4, net_model, occ4, en), reps=3)
     out["mlpnet_energy_256"] = {"ms": emsn,
