@@ -818,8 +818,6 @@ smc_status fcc_sweep_tables(const smc_lattice *lat, const smc_model *m, std::vec
 // Half-unit basis of sublattice s, and the sublattice of a half-unit parity.
 std::array<int, 3> fcc_basis(int s) { return {(s == 1 || s == 2) ? 1 : 0, (s == 1 || s == 3) ? 1 : 0, (s == 2 || s == 3) ? 1 : 0}; }
 
-int floor_half(int v) { return v >= 0 ? v / 2 : -((1 - v) / 2); }
-
 // The shell vectors in table order (shell 1: 0-11, 2: 12-17, 3: 18-41).
 std::vector<std::array<int, 3>> fcc_vectors()
 {

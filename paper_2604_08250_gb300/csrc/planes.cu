@@ -274,8 +274,6 @@ __global__ void __launch_bounds__(256) k_plane_own(const uint4 *__restrict__ pla
 
 bool g_vec_ready[64];
 
-int floor2(int v) { return v >= 0 ? v / 2 : -((1 - v) / 2); }
-
 // The vector tables of both lattices, in half units from a site of sublattice
 // s: BCC (+-1)^3, (+-2, 0, 0), (+-2, +-2, 0); FCC of squared length 2, 4, 6
 // with an even component sum.
@@ -310,8 +308,8 @@ smc_status vec_tables()
                                     for (int k = 0; k < 3; ++k) q[k] += fcc[s][k];
                                     while (fcc[ns][0] != (q[0] & 1) || fcc[ns][1] != (q[1] & 1) || fcc[ns][2] != (q[2] & 1)) ++ns;
                                 }
-                                h[lat].v[s][n++] = (uint32_t)(ns | (floor2(q[0]) + 2) << 4 | (floor2(q[1]) + 2) << 8 |
-                                                              (floor2(q[2]) + 2) << 12);
+                                h[lat].v[s][n++] = (uint32_t)(ns | (floor_half(q[0]) + 2) << 4 | (floor_half(q[1]) + 2) << 8 |
+                                                              (floor_half(q[2]) + 2) << 12);
                             }
                 if (n != shell_first(lat, m) + shell_size(lat, m)) {
                     set_error("internal error: shell vectors");

@@ -456,8 +456,6 @@ struct BccQsro {
     }
 };
 
-int bq_floor_half(int v) { return v >= 0 ? v / 2 : -((1 - v) / 2); }
-
 int bq_rows(int nsh) { return nsh == 1 ? 13 : (nsh == 2 ? 21 : 25); }
 
 // Rows that the trials of sublattice `sub` reach (row_group.cuh: the row of a,
@@ -478,8 +476,8 @@ bool bq_group_tables(int nsh, int pitch, const std::vector<uint32_t> &w, std::ve
             if (((hy ^ hz) & 1) || slot[hy + 3][hz + 3] >= 0) return;
             slot[hy + 3][hz + 3] = R.n;
             R.sub[R.n] = (signed char)((s + hy) & 1);
-            R.dy[R.n] = (signed char)bq_floor_half(s + hy);
-            R.dz[R.n] = (signed char)bq_floor_half(s + hz);
+            R.dy[R.n] = (signed char)floor_half(s + hy);
+            R.dz[R.n] = (signed char)floor_half(s + hz);
             ++R.n;
         };
         need(0, 0);
@@ -495,7 +493,7 @@ bool bq_group_tables(int nsh, int pitch, const std::vector<uint32_t> &w, std::ve
                     const int sl = slot[hy + 3][hz + 3];
                     if (sl < 0) return false;
                     out[(size_t)(kQgOff + s * kQgSub + (e < nz ? e : kQgZone) * kQgDirs + d)] =
-                        qg_pack(sl, pitch, bq_floor_half(s + hx));
+                        qg_pack(sl, pitch, floor_half(s + hx));
                 }
         if (R.nwr != 5 || R.n != bq_rows(nsh) || R.sub[0] != s) return false;
     }

@@ -136,6 +136,9 @@ __device__ __forceinline__ int ld_volatile_i32(const int *p)
     return *(volatile const int *)p;
 }
 
+// v / 2, rounded down: the cell of a half-unit coordinate.
+inline int floor_half(int v) { return v >= 0 ? v / 2 : -((1 - v) / 2); }
+
 // ---------------------------------------------------------------------------
 // Host-side internals shared by the translation units.
 // ---------------------------------------------------------------------------

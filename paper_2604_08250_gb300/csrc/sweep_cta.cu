@@ -30,7 +30,6 @@ namespace {
 
 constexpr int kCtaRing = 1024;      // ring entries per half
 constexpr int kCtaRngWarps = 4;
-constexpr int kCtaMaxCompute = 512; // compute threads
 
 // Shared-memory layout of one replica.
 struct CtaLayout {
@@ -48,7 +47,7 @@ __host__ __device__ inline CtaLayout cta_layout(int nx, int ny, int nz, int nsh)
     L.EY = ny + 4;
     L.EZ = nz + 4;
     L.ntr = (nx / Lx) * (ny / Ly) * (nz / Lz);
-    L.lpt = L.ntr <= 1 ? 32 : (L.ntr <= 2 ? 16 : (L.ntr <= 4 ? 8 : (L.ntr <= 128 ? 4 : 2)));
+    L.lpt = L.ntr <= 1 ? 32 : (L.ntr <= 2 ? 16 : (L.ntr <= 4 ? 8 : 4));
     L.cthr = (L.ntr * L.lpt + 31) / 32 * 32;
     L.E = Lx == 4 && nx % 4 == 0 ? 4 : 1;  // the four sites of a link cell's row share a Philox block
     L.units = kCtaRing / (L.ntr * L.E) > 0 ? kCtaRing / (L.ntr * L.E) : 1;
@@ -329,8 +328,7 @@ __global__ void k_sweep_cta(const __grid_constant__ SweepParams P, int check)
         case 32: cta_compute<IS_INT, NSH, 32>(P, L, RD, tid, accE, accN, rep); break;
         case 16: cta_compute<IS_INT, NSH, 16>(P, L, RD, tid, accE, accN, rep); break;
         case 8: cta_compute<IS_INT, NSH, 8>(P, L, RD, tid, accE, accN, rep); break;
-        case 4: cta_compute<IS_INT, NSH, 4>(P, L, RD, tid, accE, accN, rep); break;
-        default: cta_compute<IS_INT, NSH, 2>(P, L, RD, tid, accE, accN, rep); break;
+        default: cta_compute<IS_INT, NSH, 4>(P, L, RD, tid, accE, accN, rep); break;
         }
         if (accE) atomicAdd(&s_e, (unsigned long long)accE);
         if (accN) atomicAdd(&s_n, (unsigned long long)accN);
