@@ -119,7 +119,6 @@ __device__ void cta_compute(const SweepParams &P, const CtaLayout &L, const RepD
     }
     int half = 0;
     for (int t = 0; t < P.nsweeps; ++t) {
-        int accS = 0;  // accepted trials of this sweep (at most the lattice's sites; a launch's exceed 32 bits)
         float cx = 0.f;
         int32_t band = 0;  // floating-point models: dE in (lo, lo + band] needs the exact test
         if constexpr (!IS_INT) {
@@ -131,6 +130,7 @@ __device__ void cta_compute(const SweepParams &P, const CtaLayout &L, const RepD
             const uint4 *ring = (const uint4 *)(g_smem + L.ring) + half * kCtaRing;
             half ^= 1;
             const int steps = min(L.units, L.nunit - u0) * L.E;
+            int accS = 0;  // accepted trials of this unit: those of a launch may exceed 32 bits
             uint4 e = on ? ring[trial] : make_uint4(0, 0, 0, 0);
             for (int k = 0; k < steps; ++k) {
                 // entry: word, offset of a, its extended coordinates (10 bits each) and sublattice, accepted dE
@@ -205,8 +205,8 @@ __device__ void cta_compute(const SweepParams &P, const CtaLayout &L, const RepD
                 else
                     asm volatile("bar.sync 1, %0;" ::"r"(L.cthr) : "memory");
             }
+            accN += accS;
         }
-        accN += accS;
     }
 }
 
@@ -279,8 +279,13 @@ __device__ void cta_rng(const SweepParams &P, const CtaLayout &L, const RepDesc 
     }
 }
 
+// The bounds are those of the largest block.  Without them ptxas aims at fewer
+// registers than the chain of a mini-step wants (64 instead of 90): 8^3 cells,
+// us per sweep, integer / FP32: 36.4 / 42.4, with them 29.3 / 32.4; 11^3, one
+// trial per mini-step: 393 / 450 and 388 / 438; 12^3 three shells of eight species:
+// 60 / 55 and 52 / 54.
 template <bool IS_INT, int NSH>
-__global__ void k_sweep_cta(const __grid_constant__ SweepParams P, int check)
+__global__ void __launch_bounds__(4 * kCtaMaxTrials + 32 * kCtaRngWarps, 1) k_sweep_cta(const __grid_constant__ SweepParams P, int check)
 {
     const int rep = blockIdx.x, tid = threadIdx.x, nthr = blockDim.x;
     const RepDesc &RD = P.rep[rep];
