@@ -14,9 +14,9 @@
 //
 // One thread per trial.  Rows of up to 1024 cells run the four mini-steps of a
 // group in one launch on rows in shared memory (k_fcc_group here,
-// k_qsro_group in qsro_group.cuh; 256^3 cells, 2 shells: 41 us per group of
-// the pair model and 92 of the qSRO model, against 91 and 188 with a launch
-// per mini-step; 128^3: 13 and 22 against 66 and 104).  Longer rows run one
+// k_qsro_group in qsro_group.cuh; 256^3 cells, 2 shells: 37 us per group of
+// the pair model and 93 of the qSRO model, against 91 and 188 with a launch
+// per mini-step; 128^3: 10 and 21 against 66 and 104).  Longer rows run one
 // launch per mini-step (k_fcc_ministep, k_fcc_qsro_ministep, described next):
 // the trials of a mini-step touch disjoint read and write sets (pinned
 // exhaustively on the CPU for 1-3 shells), and consecutive launches are

@@ -3,7 +3,7 @@
 // one thread per trial, the trials of a mini-step being independent
 // (read/write sets pinned on the CPU).  Rows of up to 1024 cells run the four
 // mini-steps of a group in one launch on rows in shared memory
-// (qsro_group.cuh; 256^3, 2 shells: 65 us per group against 139 with a launch
+// (qsro_group.cuh; 256^3, 2 shells: 63 us per group against 139 with a launch
 // per mini-step), longer ones k_bq_ministep, a launch per mini-step.
 //
 // Site j's energy changes only through the species of its neighbours a and

@@ -13,9 +13,10 @@
 // saves three of four launches and reads each row once for four mini-steps.
 // Rows start a multiple of 128 bytes apart in the pair kernel, so that the rows
 // that different lanes pick by their partner direction share no bank beyond
-// the cell offset (41 us per group of 256^3 FCC cells, 43 us with 32), and a
-// multiple of 64 in the qSRO kernels, which keep twice the bytes per column
-// (92 against 110 us with 128, which leaves room for fewer columns).
+// the cell offset (256^3 FCC cells, two shells, us per group: 35.1, with 64
+// 34.8, with 32 36.2; three shells 65.5, 65.5, 67.6), and a multiple of 64 in
+// the qSRO kernels, which keep twice the bytes per column (90 us, 101 with 32,
+// 104 with 128, which leaves room for fewer columns).
 #pragma once
 
 #include <algorithm>
