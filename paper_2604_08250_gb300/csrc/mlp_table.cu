@@ -689,17 +689,23 @@ __global__ void __launch_bounds__(256) k_unlike_bonds(const int8_t *__restrict__
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, (unsigned long long)n);
 }
 
-__global__ void k_table_route(TableGain gain, double bonds, const unsigned long long *unlike, int *route)
+// The choice (1: tabulated), and for the host to see (echo, pinned) with the
+// call's number: 2 call + choice.
+__global__ void k_table_route(TableGain gain, double bonds, const unsigned long long *unlike, uint32_t call, int *route,
+                              volatile uint32_t *echo)
 {
-    *route = gain.at((double)*unlike / bonds) > 0.0 ? 1 : 0;
+    const int r = gain.at((double)*unlike / bonds) > 0.0 ? 1 : 0;
+    *route = r;
+    if (echo) *echo = 2u * call + (uint32_t)r;
 }
 
-// The route word's copy on the host.  The host never waits for it: it looks
-// before it enqueues each sweep, and what was enqueued before the word came
-// ends at once where it is not needed.
+// The host never waits for the choice: it looks before it enqueues each sweep,
+// and what was enqueued before the word came ends at once where it is not
+// needed.  (A look is a load: an event query would break a capture that another
+// thread has under way.)
 struct RouteEcho {
-    int *word = nullptr;  // pinned
-    cudaEvent_t event = nullptr;
+    uint32_t *word = nullptr;  // pinned
+    uint32_t call = 0;         // 31 bits
 };
 RouteEcho *route_echo()
 {
@@ -707,11 +713,16 @@ RouteEcho *route_echo()
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return nullptr;
     RouteEcho &r = echo[dev];
-    if (!r.word && cudaHostAlloc((void **)&r.word, sizeof(int), cudaHostAllocDefault) != cudaSuccess) r.word = nullptr;
-    if (!r.event && cudaEventCreateWithFlags(&r.event, cudaEventDisableTiming) != cudaSuccess) r.event = nullptr;
-    if (r.word && r.event) return &r;
-    cudaGetLastError();
-    return nullptr;
+    if (!r.word) {
+        if (cudaHostAlloc((void **)&r.word, sizeof(uint32_t), cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();
+            r.word = nullptr;
+            return nullptr;
+        }
+        *r.word = 0;
+    }
+    r.call = (r.call + 1) & 0x7FFFFFFFu;
+    return &r;
 }
 
 }  // namespace
@@ -802,23 +813,18 @@ smc_status launch_mlp_table_sweep(const smc_lattice *lat, const smc_model *m, in
             k_unlike_bonds<true><<<cb, 256, 0, stream>>>(occ, P.nx, P.ny, P.nz, unlike);
         else
             k_unlike_bonds<false><<<cb, 256, 0, stream>>>(occ, P.nx, P.ny, P.nz, unlike);
-        k_table_route<<<1, 1, 0, stream>>>(gain, 4.0 * (double)N, unlike, word);
+        echo = route_echo();
+        k_table_route<<<1, 1, 0, stream>>>(gain, 4.0 * (double)N, unlike, echo ? echo->call : 0u, word,
+                                           echo ? echo->word : nullptr);
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "k_table_route");
         P.route = *route = word;
-        echo = route_echo();
-        if (echo) {
-            e = cudaMemcpyAsync(echo->word, word, sizeof(int), cudaMemcpyDeviceToHost, stream);
-            if (e == cudaSuccess) e = cudaEventRecord(echo->event, stream);
-            if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(route)");
-        }
     }
     // looks whether the route is known by now; false: the rest of the tabulated sweep is not needed
     auto go_on = [&]() {
         if (*taken != kMlpEither || !echo) return true;
-        const cudaError_t q = cudaEventQuery(echo->event);
-        if (q == cudaErrorNotReady) cudaGetLastError();
-        if (q == cudaSuccess) *taken = *(volatile int *)echo->word ? kMlpTabulate : kMlpEvaluate;
+        const uint32_t w = *(volatile uint32_t *)echo->word;
+        if (w >> 1 == echo->call) *taken = w & 1u ? kMlpTabulate : kMlpEvaluate;
         return *taken != kMlpEvaluate;
     };
     st = mlp_copy_weights(m, scr + o_w, stream);
