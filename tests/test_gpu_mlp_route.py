@@ -133,3 +133,32 @@ def test_occupancy_at_any_address(smc):
         smc.sweep(lat, model, at, 7, 2, 24, KT)
         smc.check()
         assert torch.equal(at, want)
+
+
+def test_call_while_another_thread_captures(smc):
+    import threading
+    lat, occ = _alloy(smc, (96, 96, 96), FRACTIONS[1])
+    model = _model(smc, "mlp", 5)
+    want, _, _ = _sweep(smc, lat, model, occ, 24, route=1)
+    _sweep(smc, lat, model, occ, 24)  # its buffers
+    got, errors = occ.clone(), []
+    torch.cuda.synchronize()
+
+    def call():
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                smc.sweep(lat, model, got, 7, 2, 24, KT)
+        except Exception as err:  # noqa: BLE001
+            errors.append(err)
+    x = torch.ones(8, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        y = x + 1
+        t = threading.Thread(target=call)
+        t.start()
+        t.join()
+        z = y * 2
+    g.replay()
+    torch.cuda.synchronize()
+    smc.check()
+    assert not errors and torch.equal(got, want) and float(z.sum()) == 32.0
