@@ -42,6 +42,36 @@ print("ok")
 """
 
 
+WORKSPACE = """
+import torch
+from paper_2604_08250_gb300 import inputs, smc
+lat = smc.Lattice(256, 128, 128, 5)
+occ = torch.zeros(lat.nsites, dtype=torch.int8, device="cuda")
+model = smc.Model(smc.MLP_BF16, mlp=inputs.mlp_weights(3))
+smc.debug_set(smc.DBG_MLP_TABLE, 1)
+smc.energy(lat, model, occ, torch.zeros(1, dtype=torch.float64, device="cuda"))  # the kernels are loaded
+small = smc.Lattice(16, 16, 16, 5)
+smc.sweep(small, model, occ[:small.nsites], 1, 0, 1, 0.07)
+torch.cuda.synchronize()
+f0 = torch.cuda.mem_get_info()[0]
+smc.sweep(lat, model, occ, 1, 0, 1, 0.07)
+torch.cuda.synchronize()
+kept, need = f0 - torch.cuda.mem_get_info()[0], 20 * lat.nsites
+assert need <= kept + (4 << 20) and kept <= need + (8 << 20), (kept, need)
+print("ok")
+"""
+
+
+def test_large_workspaces_grow_to_what_is_needed():
+    """20 bytes per site of an MLP sweep's caches and little more, not the next power of two."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2604_08250_gb300 import build
+    build.build()
+    r = subprocess.run([sys.executable, "-c", WORKSPACE], cwd=build.ROOT, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
+
+
 def test_memory_that_a_tabulated_sweep_keeps():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
