@@ -1106,7 +1106,6 @@ smc_status launch_mlp_trace(const smc_lattice *lat, const smc_model *m, int8_t *
 // qSRO host side.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr double kShellZ[3] = {8.0, 6.0, 12.0};
 
 QsroRaw make_qsro_raw(const smc_model *m, int S)
 {
